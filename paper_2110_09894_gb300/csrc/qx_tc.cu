@@ -201,6 +201,26 @@ __device__ __forceinline__ void mbar_wait_issued(uint64_t* b, uint32_t parity) {
     while (!mbar_try(b, parity))
         if (clock64() - t0 > kIssuedWaitCycles) return;
 }
+// progress of another warp of the CTA: waits (bounded as mbar_wait) until *p has reached `stage`; stage
+// numbers compare modulo 2^32
+__device__ __forceinline__ void prog_set(int* p, int stage) {
+    asm volatile("st.release.cta.shared::cta.b32 [%0], %1;" ::"r"(s_addr(p)), "r"(stage) : "memory");
+}
+__device__ __forceinline__ bool prog_wait(const int* p, int stage, long long limit, const int* err) {
+    auto reached = [&]() {
+        int v;
+        asm volatile("ld.acquire.cta.shared::cta.b32 %0, [%1];" : "=r"(v) : "r"(s_addr(p)) : "memory");
+        return (int)((uint32_t)v - (uint32_t)stage) >= 0;
+    };
+    if (reached()) return true;
+    const long long t0 = clock64();
+    uint32_t spins = 0;
+    while (!reached()) {
+        if (clock64() - t0 > limit) return false;
+        if ((++spins & 1023) == 0 && *(volatile const int*)err) return false;
+    }
+    return true;
+}
 __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, int c0, int c1, int c2, uint64_t* bar) {
     asm volatile(
         "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], "
@@ -677,6 +697,7 @@ __global__ void __launch_bounds__(TC2_THREADS2, 1)
     __shared__ uint64_t full[NL], lfree[NL], mfull[NM], mfree[NM], tfull[NTB], tempty[NTB], drain[2];
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
+    __shared__ int conv_seen[2][4];  // per converter group and warp: the last stage whose slots it saw ready
     if (*(volatile const int*)err) return;
     uint8_t* base = (uint8_t*)(((uintptr_t)dyn + 1023) & ~(uintptr_t)1023);
     auto land = [&](int l) { return base + l * L::LAND; };
@@ -713,6 +734,7 @@ __global__ void __launch_bounds__(TC2_THREADS2, 1)
         }
         mbar_init(&drain[0], 1);
         mbar_init(&drain[1], 1);
+        for (int w = 0; w < 8; ++w) conv_seen[w >> 2][w & 3] = -1;
         abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -773,8 +795,12 @@ __global__ void __launch_bounds__(TC2_THREADS2, 1)
         uint32_t mph = 0;
         int64_t u = 0;  // g / NTB
         for (int64_t g = who; g < total && ok; g += 2, ++u) {
-            if (!mbar_wait(&mfull[m], mph, limit, err) ||
-                (u > 0 && !mbar_wait(&tempty[b], (uint32_t)((u - 1) & 1), limit, err)) || *(volatile int*)&abort_flag) {
+            // the accumulator first: it is free once stage g - 2, and with it every stage before, was
+            // drained, so the slot's earlier uses (stage g - NM may be the other issuer's) are over and
+            // the parity below can only mean this stage.  The other way round, an issuer ahead of a
+            // late stage g - NM would take that slot's last phase for its own and read it unconverted.
+            if ((u > 0 && !mbar_wait(&tempty[b], (uint32_t)((u - 1) & 1), limit, err)) ||
+                !mbar_wait(&mfull[m], mph, limit, err) || *(volatile int*)&abort_flag) {
                 atomicExch(&abort_flag, 1);
                 ok = false;
                 break;
@@ -821,13 +847,19 @@ __global__ void __launch_bounds__(TC2_THREADS2, 1)
         int64_t t = grp / nk, prev_key = -1;
         bool with_a = true;
         for (int64_t g = grp; g < total; g += ng) {
-            // one decision per warp: the TMEM stores of the conversion are warp-wide (.sync.aligned)
-            const bool go = mbar_wait(&full[l], lph, limit, err) && mbar_wait(&mfree[m], mph ^ 1u, limit, err) &&
+            // one decision per warp: the TMEM stores of the conversion are warp-wide (.sync.aligned).
+            // With two groups a slot's uses alternate between them, and a parity alone cannot tell a
+            // phase from the one two before: the other group's warp must have seen stage g - 3 first
+            // (then the slots' uses before the last are over; g itself has to wait for that stage's
+            // slot in any case).
+            const bool go = (ng == 1 || g < 3 || prog_wait(&conv_seen[grp ^ 1][warp & 3], (int)(g - 3), limit, err)) &&
+                            mbar_wait(&full[l], lph, limit, err) && mbar_wait(&mfree[m], mph ^ 1u, limit, err) &&
                             !*(volatile int*)&abort_flag;
             if (!__all_sync(0xffffffffu, go)) {
                 atomicExch(&abort_flag, 1);
                 break;
             }
+            if (ng == 2 && lane == 0) prog_set(&conv_seen[grp][warp & 3], (int)g);
             if (keep_a && it == 0) {
                 int64_t item, akey;
                 int m0, n0;
@@ -835,12 +867,12 @@ __global__ void __launch_bounds__(TC2_THREADS2, 1)
                 with_a = akey != prev_key;
                 prev_key = akey;
                 if (with_a && g > 0) {
-                    // a new A overwrites the kept one: every MMA of the earlier stages must be done
-                    // (each stage's commit to its accumulator buffer covers the MMAs its issuer issued
-                    // before it)
+                    // a new A overwrites the kept one: every MMA of the earlier stages must be done.  The
+                    // wait above covers stage g - NM; each later stage's slot is freed by the commit
+                    // after its MMAs, and its next use is not yet converted.
                     bool ok = true;
-                    for (int64_t p = g - 1; p >= 0 && p >= g - 2 && ok; --p)
-                        ok = mbar_wait(&tfull[p & 1], (uint32_t)((p >> 1) & 1), limit, err);
+                    for (int64_t p = g - 1; p >= 0 && p > g - NM && ok; --p)
+                        ok = mbar_wait(&mfree[p % NM], (uint32_t)((p / NM) & 1), limit, err);
                     if (!__all_sync(0xffffffffu, ok)) {
                         atomicExch(&abort_flag, 1);
                         break;
@@ -1219,8 +1251,9 @@ __global__ void __launch_bounds__(TC2_THREADS, 1)
         uint32_t mph = 0;
         int64_t u = 0;
         for (int64_t g = who; g < total && ok; g += 2, ++u) {
-            if (!mbar_wait(&mfull[m], mph, limit, err) ||
-                (u > 0 && !mbar_wait(&tempty[b], (uint32_t)((u - 1) & 1), limit, err)) || *(volatile int*)&abort_flag) {
+            // the accumulator first (see k_gemm_tc2: the slot's earlier uses are then over)
+            if ((u > 0 && !mbar_wait(&tempty[b], (uint32_t)((u - 1) & 1), limit, err)) ||
+                !mbar_wait(&mfull[m], mph, limit, err) || *(volatile int*)&abort_flag) {
                 atomicExch(&abort_flag, 1);
                 ok = false;
                 break;
