@@ -13,6 +13,20 @@ constexpr int kSmallMaxK = 5;  // shared bits handled by the gather kernel
 constexpr int kSmallMaxN = 5;  // free bits of its small operand
 constexpr int kMaxBatchItems = 65535;
 
+#ifdef __CUDACC__
+// One term of a Neumaier sum: s + x rounded into s, its rounding error added to c.  The error is
+// (larger - t) + smaller by magnitude; the comparison looks at the bit patterns (magnitudes order
+// like their bits) so that only the four additions use the FP64 unit, which adds about two doubles a
+// clock per SM.
+__device__ __forceinline__ void neumaier(double& s, double& c, double x) {
+    const double t = s + x;
+    const bool keep = (__double_as_longlong(s) & 0x7fffffffffffffffll) >= (__double_as_longlong(x) & 0x7fffffffffffffffll);
+    const double big = keep ? s : x, small = keep ? x : s;
+    c += (big - t) + small;
+    s = t;
+}
+#endif
+
 // The (slice, bitstring) pairs of one batch: item = s_local * n_b + b_local.
 struct ItemCtx {
     int64_t s0;            // first slice of the batch

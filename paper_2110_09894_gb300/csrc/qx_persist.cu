@@ -329,53 +329,60 @@ __global__ void __launch_bounds__(256, 2) k_persist(const PLaunch L) {
     }
 }
 
-__device__ __forceinline__ void neumaier_add(double& s, double& c, double x) {
-    const double t = s + x;
-    if (fabs(s) >= fabs(x)) c += (s - t) + x;
-    else c += (x - t) + s;
-    s = t;
-}
-
-__device__ __forceinline__ void gsum_one(const GSum& g, int64_t local) {
-    const int64_t n_o = (int64_t)1 << g.open_bits;
-    const int64_t b = local >> g.open_bits, o = local & (n_o - 1);
-    double sr = 0, si = 0, cr = 0, ci = 0;
-    for (int s = 0; s < g.n_s; ++s) {
-        const float2 v = g.results[((int64_t)s * g.n_b + b) * n_o + o];
-        neumaier_add(sr, cr, (double)v.x);
-        neumaier_add(si, ci, (double)v.y);
+// One thread per component of an amplitude (see k_slice_sum: the FP64 unit is the limit, so one warp
+// per CTA, loads ahead of the additions, slices in order).  local2 = 2 * amplitude + component.
+constexpr int kSumThreads = 32, kSumAhead = 16;
+__device__ __forceinline__ void gsum_one(const GSum& g, int64_t local2, bool live) {
+    const int64_t local = local2 >> 1, n_o = (int64_t)1 << g.open_bits;
+    const int c = (int)(local2 & 1);
+    double s = 0, comp = 0;
+    if (live) {
+        // result of slice i: [i][bitstring][open index]; local = bitstring * n_o + open index
+        const float* p = (const float*)(g.results + local) + c;
+        const int64_t step = 2 * g.n_b * n_o;
+        int i = 0;
+        for (; i + kSumAhead <= g.n_s; i += kSumAhead) {
+            float v[kSumAhead];
+#pragma unroll
+            for (int k = 0; k < kSumAhead; ++k) v[k] = p[(i + k) * step];
+#pragma unroll
+            for (int k = 0; k < kSumAhead; ++k) neumaier(s, comp, (double)v[k]);
+        }
+        for (; i < g.n_s; ++i) neumaier(s, comp, (double)p[i * step]);
     }
-    const double re = sr + cr, im = si + ci;
-    g.amps[2 * local] = re * g.sr - im * g.si;
-    g.amps[2 * local + 1] = re * g.si + im * g.sr;
+    const double mine = s + comp, other = __shfl_xor_sync(0xffffffffu, mine, 1);
+    if (!live) return;
+    if (c == 0) g.amps[2 * local] = mine * g.sr - other * g.si;
+    else g.amps[2 * local + 1] = other * g.si + mine * g.sr;
 }
 
-__global__ void k_group_sum(const GSum* __restrict__ sums, int32_t n, int64_t total) {
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= total) return;
+__global__ void __launch_bounds__(kSumThreads) k_group_sum(const GSum* __restrict__ sums, int32_t n, int64_t total) {
+    const int64_t t2 = (int64_t)blockIdx.x * kSumThreads + threadIdx.x;
+    const bool live = t2 < 2 * total;
+    const int64_t t = live ? t2 >> 1 : 0;
     int lo = 0, hi = n - 1;  // last program with t0 <= t
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
         if (sums[mid].t0 <= t) lo = mid;
         else hi = mid - 1;
     }
-    gsum_one(sums[lo], t - sums[lo].t0);
+    gsum_one(sums[lo], t2 - 2 * sums[lo].t0, live);
 }
 
-__global__ void k_single_sum(const GSum g, int64_t total) {
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < total) gsum_one(g, t);
+__global__ void __launch_bounds__(kSumThreads) k_single_sum(const GSum g, int64_t total) {
+    const int64_t t2 = (int64_t)blockIdx.x * kSumThreads + threadIdx.x;
+    gsum_one(g, t2, t2 < 2 * total);
 }
 
 cudaError_t launch_single_sum(const GSum& g, int64_t total, cudaStream_t st) {
     if (total <= 0) return cudaSuccess;
-    k_single_sum<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(g, total);
+    k_single_sum<<<(unsigned)((2 * total + kSumThreads - 1) / kSumThreads), kSumThreads, 0, st>>>(g, total);
     return cudaGetLastError();
 }
 
 cudaError_t launch_group_sum(const GSum* d_sums, int32_t n, int64_t total, cudaStream_t st) {
     if (total <= 0 || n <= 0) return cudaSuccess;
-    k_group_sum<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(d_sums, n, total);
+    k_group_sum<<<(unsigned)((2 * total + kSumThreads - 1) / kSumThreads), kSumThreads, 0, st>>>(d_sums, n, total);
     return cudaGetLastError();
 }
 
