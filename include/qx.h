@@ -266,9 +266,11 @@ int qx_set_memo(qx_handle h, int enable);
  * captured graph. */
 int qx_set_streams(qx_handle h, int32_t n_streams);
 
-/* A text listing of the compiled plan, one line per kernel launch of a
- * contraction (kind, whether it runs per pair or once, M/K/N bits, operand
- * layouts).  Writes at most len bytes (NUL-terminated) to buf; *needed (may be
+/* A text listing of the compiled plan, one line per step's kernel (kind,
+ * whether it runs per pair or once, M/K/N bits, operand layouts).  Steps with
+ * the same chain= or seg= number may run as one launch: chains in the
+ * prologue launch of a call, segments where one launch is the faster way for
+ * the call's items.  Writes at most len bytes (NUL-terminated) to buf; *needed (may be
  * NULL) receives the full size.  Works on host-only handles. */
 int qx_describe_plan(qx_handle h, char* buf, int64_t len, int64_t* needed);
 
@@ -403,7 +405,7 @@ void qx_group_destroy(qx_group_t g);
 #define QX_KERNEL_TC_PREP 4  /* operand split / expansion for the tensor-core forms */
 #define QX_KERNEL_TC_GEMM 5  /* tcgen05 complex GEMM on pre-split operands (k_gemm_tc) */
 #define QX_KERNEL_PERSIST 6  /* persistent executor (whole contractions) */
-#define QX_KERNEL_WAVE    7  /* batched executor: the small invariant steps, one CTA per chain */
+#define QX_KERNEL_WAVE    7  /* batched executor: connected groups of small steps in one launch (k_seg) */
 #define QX_KERNEL_SMALL_FLAT 8  /* gathers of short per-pair rows, one thread per row (k_small_flat) */
 #define QX_KERNEL_TC_DIRECT 9  /* tcgen05 3xTF32 GEMM splitting raw complex64 slabs itself (k_gemm_tc2) */
 #define QX_KERNEL_TC_DIRECT_KB 10  /* the same with B' built once per CTA and kept (k_gemm_tc2kb): B

@@ -14,6 +14,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <array>
 #include <cmath>
 #include <cstdarg>
 #include <cstdint>
@@ -22,11 +23,13 @@
 #include <functional>
 #include <limits>
 #include <map>
+#include <memory>
 #include <string>
 #include <vector>
 
 #include "qx.h"
 #include "qx_internal.h"
+#include "qx_seg.h"
 
 using namespace qx;
 
@@ -94,6 +97,8 @@ struct Op {
     double flops = 0;
 };
 
+struct SegPlan;
+
 }  // namespace
 
 struct qx_ctx {
@@ -140,17 +145,33 @@ struct qx_ctx {
     int persist_grid = 0;
     bool pops_on_device = false;
 
-    // batched executor prologue: the invariant steps as chains that share no storage, one launch,
-    // one CTA per chain (only when every invariant step is small)
-    bool wave_ok = false;
-    std::vector<POp> wave_ops;          // one per invariant op, grouped by chain
-    std::vector<int32_t> wave_idx;      // 0 .. n-1 (positions into wave_ops)
-    std::vector<int32_t> wave_start;    // chain c: wave_ops[wave_start[c] .. wave_start[c + 1])
-    std::vector<int> wave_of;           // per op: 0 if the prologue launch runs it, else -1
-    std::vector<int> chain_of_op;       // per op: its prologue chain, -1 if none
-    std::vector<double> wave_flops, wave_bytes;
-    bool waves_on_device = false;
-    std::vector<cudaEvent_t> wave_ev;
+    // batched executor: segments, connected groups of small steps of one level that one launch runs
+    // with their intermediates in shared memory (k_seg).  The invariant segments that read only leaves
+    // run together in one prologue launch (wave_*).
+    struct Seg {
+        int level = 0;
+        bool wave = false;             // runs in the prologue launch
+        std::vector<int> ops;          // plan order; the last one is the root
+        std::shared_ptr<SegPlan> plan;
+        int n_stages = 0, n_tasks = 0, arena = 0;
+        double warp_clocks = 0;        // estimated issue clocks of one item's tasks
+        double bytes = 0;              // of its steps as launches of their own, per item
+        double flops = 0;
+        int64_t prog_off = 0;          // bytes into seg_blob
+        int32_t prog_bytes = 0;
+    };
+    std::vector<Seg> segs;
+    std::vector<int> seg_of;            // per op: its segment, -1 if none
+    std::vector<uint8_t> seg_blob;      // the programs, then the prologue programs' offsets
+    int64_t wave_list = 0;              // byte offset of those offsets in seg_blob
+    int n_waves = 0;
+    bool segs_on = true;                // false: every step a launch of its own (workspaces too small for segments)
+    std::vector<Storage> stor0;         // storages with the lifetimes of one launch per step
+    bool wave_ok = false;               // there is a prologue launch
+    std::vector<int> chain_of_op;       // per op: its prologue segment, -1 if none
+    double wave_flops = 0, wave_bytes = 0;
+    bool segs_on_device = false;
+    cudaEvent_t wave_ev = nullptr;
 
     // workspace
     char* ws = nullptr;
@@ -450,7 +471,9 @@ static int64_t assign_offsets(qx_ctx* h, int level) {
 }
 
 static void build_persistent_program(qx_ctx* h);
-static void build_waves(qx_ctx* h);
+static void choose_segments(qx_ctx* h);
+static void build_segments(qx_ctx* h);
+static void finish_layout(qx_ctx* h, bool segs);
 
 // Storages an op reads and writes (leaves are read-only and not listed), and whether it uses the
 // per-tensor scale words of the workspace (prep-based tensor-core steps).
@@ -1084,11 +1107,26 @@ static int compile_plan(qx_ctx* h, const int64_t* order, int64_t n_steps, const 
             else keep_stor(op.sb);
         }
     }
+    h->stor0 = h->stor;
+    finish_layout(h, true);
+    h->flops_inv = h->flops_slice = h->flops_item = 0;
+    for (const Op& op : h->ops) (op.level == 2 ? h->flops_item : op.level == 1 ? h->flops_slice : h->flops_inv) += op.flops;
+    h->have_plan = true;
+    return QX_OK;
+}
+
+// Offsets, dependencies and programs of the compiled ops.  segs: small steps grouped into segments,
+// whose operands from outside live until the segment's last step (and whose results in the prologue
+// live from the start); without them every step is a launch of its own, which needs the least memory.
+static void finish_layout(qx_ctx* h, bool segs) {
+    h->segs_on = segs && h->opt.executor < 2;
+    h->stor = h->stor0;
+    choose_segments(h);
     h->item_entries = std::max<int64_t>(assign_offsets(h, 2), kAlignEntries);
     h->slice_entries = assign_offsets(h, 1);
     if (h->opt.executor < 2) {
         // a small invariant region gets no reuse: then the only hazards between invariant steps are
-        // their data dependencies, which form trees the prologue runs one CTA per tree
+        // their data dependencies
         int64_t tot = 0;
         for (const Storage& st : h->stor)
             if (st.level == 0) tot += align_up(st.entries, kAlignEntries);
@@ -1100,13 +1138,9 @@ static int compile_plan(qx_ctx* h, const int64_t* order, int64_t n_steps, const 
                 }
     }
     h->inv_entries = assign_offsets(h, 0);
-    h->flops_inv = h->flops_slice = h->flops_item = 0;
-    for (const Op& op : h->ops) (op.level == 2 ? h->flops_item : op.level == 1 ? h->flops_slice : h->flops_inv) += op.flops;
     compute_deps(h);
     build_persistent_program(h);
-    build_waves(h);
-    h->have_plan = true;
-    return QX_OK;
+    build_segments(h);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1151,11 +1185,8 @@ static void layout(qx_ctx* h, int64_t max_bits, int64_t* fixed_bytes) {
         h->off_pscratch = off;
         off += align_up((int64_t)h->persist_grid * h->item_entries * 8, 256);
     }
-    h->off_wave = off;  // prologue programs: the POps, their index list, the chain boundaries
-    if (h->wave_ok)
-        off += align_up((int64_t)(h->wave_ops.size() * sizeof(POp)), 256) +
-               align_up((int64_t)(h->wave_idx.size() * sizeof(int32_t)), 256) +
-               align_up((int64_t)(h->wave_start.size() * sizeof(int32_t)), 256);
+    h->off_wave = off;  // segment programs
+    off += align_up((int64_t)h->seg_blob.size(), 256);
     h->off_slice = h->off_item = off;
     *fixed_bytes = off;
 }
@@ -1180,6 +1211,21 @@ static bool fit_regions(const qx_ctx* h, int64_t avail, int64_t max_bits, int64_
     *items_out = items;
     *slices_out = slices;
     return true;
+}
+
+// Lays out a workspace of `bytes` bytes (batch_bytes: its batch regions are a buffer of their own), with
+// segments where that fits, else with every step a launch of its own, which needs less memory.  Leaves
+// the handle in the layout that it returns the sizes of.
+static bool fit_layout(qx_ctx* h, int64_t bytes, const int64_t* batch_bytes, int64_t max_bits, int64_t* fixed,
+                       int64_t* items, int64_t* slices) {
+    for (bool segs : {true, false}) {
+        if (h->opt.executor < 2 && h->segs_on != segs) finish_layout(h, segs);
+        layout(h, max_bits, fixed);
+        const bool room = !batch_bytes || *fixed <= bytes;
+        if (room && fit_regions(h, batch_bytes ? *batch_bytes : bytes - *fixed, max_bits, items, slices)) return true;
+        if (h->opt.executor >= 2) return false;
+    }
+    return false;
 }
 
 // Region offsets for a workspace whose fixed part ends at `fixed`.
@@ -1389,71 +1435,372 @@ static void build_persistent_program(qx_ctx* h) {
 
 static double op_bytes(const qx_ctx* h, const Op& op, int64_t n_items, int64_t n_b = 1);
 
-// The invariant steps grouped into chains for the one prologue launch: steps joined by a dependency
-// (data, or space reuse where the invariant region reuses space) share a chain, which one CTA runs in
-// plan order.  Used when every invariant step is small enough for one CTA: at most 2^12 entries in
-// and out, no tensor cores, natural layouts.
-static void build_waves(qx_ctx* h) {
-    h->wave_ok = false;
-    h->wave_ops.clear();
-    h->wave_idx.clear();
-    h->wave_start.clear();
-    h->wave_flops.clear();
-    h->wave_bytes.clear();
-    h->wave_of.assign(h->ops.size(), -1);
-    h->chain_of_op.assign(h->ops.size(), -1);
-    if (h->opt.executor >= 2) return;  // the persistent executors run their own prologue program
-    constexpr int64_t kWaveEntries = 4096;
-    std::vector<int> inv;
-    for (size_t j = 0; j < h->ops.size(); ++j) {
-        const Op& op = h->ops[j];
-        if (op.variant) continue;
-        if (op.tc || !op.out_pos.empty() || op.dot_perm || h->stor[op.dst].entries > kWaveEntries) return;
-        auto small_node = [&](int n) { return node_entries(h->nodes[n]) <= kWaveEntries; };
-        if (op.type == OP_PERM && !small_node(op.src)) return;
-        if (op.type == OP_SMALL && !(small_node(op.x) && small_node(op.y))) return;
-        if (op.type == OP_GEMM &&
-            !(h->stor[op.sa].entries <= kWaveEntries && h->stor[op.sb].entries <= kWaveEntries))
-            return;
-        inv.push_back((int)j);
+// ------------------------------------------------------------------------------------------------
+// Segments: connected groups of small steps of one level, run by one launch (qx_seg.cu)
+// ------------------------------------------------------------------------------------------------
+constexpr int kSegOps = 200;               // steps of one segment
+constexpr int64_t kSegArena[3] = {12288, 4096, 4096};  // arena entries by level (8 bytes each)
+constexpr int kSegBits[3] = {12, 10, 10};  // largest tensor
+constexpr int kSegMacs[3] = {17, 14, 14};  // largest step, log2 of M K N
+
+// operand `side` (0: X / A, 1: Y / B) of an op: its node (gathers, permutes) or storage (GEMM), -1 if none
+static int seg_storage(const qx_ctx* h, const Op& op, int side) {
+    if (op.type == OP_GEMM) return side ? op.sb : op.sa;
+    const int node = op.type == OP_PERM ? (side ? -1 : op.src) : side ? op.y : op.x;
+    return node < 0 || h->nodes[node].leaf ? -1 : h->nodes[node].storage;
+}
+static int seg_operand_bits(const qx_ctx* h, const Op& op, int side) {
+    if (op.type == OP_GEMM) return op.kb + (side ? op.nb : op.mb);
+    if (op.type == OP_PERM) return side ? 0 : (int)h->nodes[op.src].legs.size();
+    return (int)h->nodes[side ? op.y : op.x].legs.size();
+}
+
+static bool seg_able(const qx_ctx* h, const Op& op) {
+    if (op.tc || op.dot_perm) return false;
+    const int lim = kSegBits[op.level];
+    if (h->stor[op.dst].entries > ((int64_t)1 << lim)) return false;
+    for (int side = 0; side < 2; ++side)
+        if (seg_operand_bits(h, op, side) > lim) return false;
+    if (op.type != OP_PERM && op.mb + op.kb + op.nb > kSegMacs[op.level]) return false;
+    // a per-slice matrix times per-pair vectors runs as one product per slice (run_op)
+    if (op.type == OP_GEMM && op.nb == 0 && op.level == 2 && h->stor[op.sa].level == 1) return false;
+    for (int side = 0; side < 2; ++side) {
+        const int node = op.type == OP_GEMM ? -1 : op.type == OP_PERM ? (side ? -1 : op.src) : side ? op.y : op.x;
+        if (node < 0) continue;
+        if ((int)h->nodes[node].fix.size() > kSegFix) return false;
+        for (auto& f : h->nodes[node].fix)
+            if (f.second > INT32_MAX) return false;
     }
-    if (inv.empty()) return;
-    // chains: invariant steps joined by a dependency (data, or space reuse when the region is
-    // reused) go to one chain, which one CTA runs in plan order; different chains touch no common
-    // storage, so the CTAs need no synchronisation
-    std::vector<int> root(h->ops.size());
-    for (size_t j = 0; j < root.size(); ++j) root[j] = (int)j;
-    std::function<int(int)> find = [&](int x) { return root[x] == x ? x : root[x] = find(root[x]); };
-    for (int j : inv)
-        for (int i : h->deps[j])
-            if (!h->ops[i].variant) root[find(i)] = find(j);
-    std::vector<int> chain_of(h->ops.size(), -1), order;
-    for (int j : inv) {
-        const int r = find(j);
-        if (chain_of[r] < 0) {
-            chain_of[r] = (int)order.size();
-            order.push_back(r);
+    return true;
+}
+
+// The arena of a segment: which operands come from outside, the steps' stages (depth), and where
+// every tensor lies (first fit over the stages it is alive in).
+namespace {
+struct SegPlan {
+    std::vector<int> stage;                       // per step
+    std::vector<std::array<int, 2>> src;          // per step and side: tensor id (operand), -1 none
+    struct Tensor { int op = -1, side = 0, bits = 0, def = 0, last = 0, off = 0; bool once = false; };
+    std::vector<Tensor> in, made;                 // operands from outside; results (made[i]: step i's)
+    int n_stages = 0, arena = 0, n_tiny = 0;
+};
+}  // namespace
+static SegPlan seg_plan(const qx_ctx* h, const std::vector<int>& ops, const std::vector<int>& producer) {
+    SegPlan p;
+    const int n = (int)ops.size(), level = h->ops[ops[0]].level;
+    auto index_of = [&](int op) {  // position in ops (plan order), -1 if not there
+        const auto it = std::lower_bound(ops.begin(), ops.end(), op);
+        return it != ops.end() && *it == op ? (int)(it - ops.begin()) : -1;
+    };
+    p.stage.assign(n, 0);
+    p.src.assign(n, {-1, -1});
+    p.made.resize(n);
+    for (int i = 0; i < n; ++i) {
+        const Op& op = h->ops[ops[i]];
+        for (int side = 0; side < (op.type == OP_PERM ? 1 : 2); ++side) {
+            const int sid = seg_storage(h, op, side);
+            const int from = sid >= 0 && producer[sid] >= 0 ? index_of(producer[sid]) : -1;
+            if (from >= 0) {
+                p.stage[i] = std::max(p.stage[i], p.stage[from] + 1);
+                p.src[i][side] = from;
+                continue;
+            }
+            SegPlan::Tensor t;
+            t.op = i;
+            t.side = side;
+            t.bits = seg_operand_bits(h, op, side);
+            t.def = -1;
+            const int node = op.type == OP_GEMM ? -1 : op.type == OP_PERM ? op.src : side ? op.y : op.x;
+            t.once = sid >= 0 ? h->stor[sid].level < level && h->stor[sid].level == 0
+                              : node >= 0 && h->nodes[node].fix.empty();
+            p.src[i][side] = n + (int)p.in.size();
+            p.in.push_back(t);
+        }
+        p.n_stages = std::max(p.n_stages, p.stage[i] + 1);
+    }
+    // tiny operands first (the kernel loads them several at a time)
+    std::vector<int> by(p.in.size()), where(p.in.size());
+    for (size_t i = 0; i < by.size(); ++i) by[i] = (int)i;
+    std::stable_partition(by.begin(), by.end(), [&](int i) { return p.in[i].bits <= 4; });
+    std::vector<SegPlan::Tensor> in;
+    for (size_t i = 0; i < by.size(); ++i) {
+        where[by[i]] = (int)i;
+        in.push_back(p.in[by[i]]);
+        p.n_tiny += p.in[by[i]].bits <= 4;
+    }
+    p.in.swap(in);
+    for (auto& sr : p.src)
+        for (int& t : sr)
+            if (t >= n) t = n + where[t - n];
+    for (int i = 0; i < n; ++i) {
+        auto& m = p.made[i];
+        m.bits = 0;
+        while (((int64_t)1 << m.bits) < h->stor[h->ops[ops[i]].dst].entries) ++m.bits;
+        m.def = m.last = p.stage[i];
+        for (int side = 0; side < 2; ++side) {
+            const int t = p.src[i][side];
+            if (t < 0) continue;
+            auto& x = t < n ? p.made[t] : p.in[t - n];
+            x.last = std::max(x.last, p.stage[i]);
         }
     }
-    const int n_chains = (int)order.size();
-    h->wave_start.assign(n_chains + 1, 0);
-    h->wave_flops.assign(1, 0.0);
-    h->wave_bytes.assign(1, 0.0);
-    for (int c = 0; c < n_chains; ++c) {
-        h->wave_start[c] = (int32_t)h->wave_ops.size();
-        for (int j : inv)
-            if (chain_of[find(j)] == c) {
-                h->wave_of[j] = 0;  // one launch: every dependant waits for its end
-                h->chain_of_op[j] = c;
-                h->wave_ops.push_back(to_pop(h, h->ops[j]));
-                h->wave_flops[0] += h->ops[j].flops;
-                h->wave_bytes[0] += op_bytes(h, h->ops[j], 1);
-            }
+    // first fit over the stages, the space of tensors of earlier stages free again; a tensor that every
+    // item shares stays for all of them
+    std::vector<SegPlan::Tensor*> all;
+    for (auto& t : p.in) all.push_back(&t);
+    for (int i = 0; i + 1 < n; ++i) all.push_back(&p.made[i]);  // the root's result goes to its storage
+    for (auto* t : all)
+        if (t->once) t->def = -1, t->last = p.n_stages;
+    std::stable_sort(all.begin(), all.end(), [](auto* a, auto* b) { return a->def < b->def; });
+    std::vector<SegPlan::Tensor*> live;  // by offset
+    int stage = -2;
+    for (auto* t : all) {
+        if (t->def != stage) {
+            stage = t->def;
+            live.erase(std::remove_if(live.begin(), live.end(), [&](auto* x) { return x->last < stage; }), live.end());
+        }
+        const int need = std::max(2, 1 << t->bits);
+        int at = 0;
+        auto it = live.begin();
+        for (; it != live.end() && at + need > (*it)->off; ++it) at = (*it)->off + std::max(2, 1 << (*it)->bits);
+        t->off = at;
+        live.insert(it, t);
+        p.arena = std::max(p.arena, at + need);
     }
-    h->wave_start[n_chains] = (int32_t)h->wave_ops.size();
-    h->wave_idx.resize(h->wave_ops.size());
-    for (size_t i = 0; i < h->wave_idx.size(); ++i) h->wave_idx[i] = (int32_t)i;
-    h->wave_ok = true;
+    return p;
+}
+
+static std::vector<int> storage_producers(const qx_ctx* h) {
+    std::vector<int> producer(h->stor.size(), -1);
+    for (size_t j = 0; j < h->ops.size(); ++j) producer[h->ops[j].dst] = (int)j;
+    return producer;
+}
+
+// Groups steps into segments and gives their operands and results the lifetimes that running a whole
+// segment at its last step (the prologue's: at the start) needs.
+static void choose_segments(qx_ctx* h) {
+    h->segs.clear();
+    h->seg_of.assign(h->ops.size(), -1);
+    if (!h->segs_on) return;
+    const std::vector<int> producer = storage_producers(h);
+    std::vector<std::vector<int>> group(h->ops.size());  // by root op, plan order
+    std::vector<int64_t> flat(h->ops.size(), 0);         // entries of all its steps' operands and results
+    for (size_t j = 0; j < h->ops.size(); ++j) {
+        const Op& op = h->ops[j];
+        if (!seg_able(h, op)) continue;
+        group[j] = {(int)j};
+        flat[j] = std::max<int64_t>(2, h->stor[op.dst].entries);
+        for (int side = 0; side < 2; ++side) flat[j] += std::max(2, 1 << seg_operand_bits(h, op, side));
+        for (int side = 0; side < 2; ++side) {
+            const int sid = seg_storage(h, op, side);
+            const int i = sid >= 0 ? producer[sid] : -1;
+            if (i < 0 || group[i].empty() || h->ops[i].level != op.level) continue;
+            std::vector<int> both = group[i];
+            both.insert(both.end(), group[j].begin(), group[j].end());
+            std::sort(both.begin(), both.end());
+            // the arena of everything at once bounds the one of the stages
+            const int64_t all = flat[i] + flat[j];
+            if ((int)both.size() > kSegOps ||
+                (all > kSegArena[op.level] && seg_plan(h, both, producer).arena > kSegArena[op.level]))
+                continue;
+            flat[j] = all;
+            group[j] = both;
+            group[i].clear();
+        }
+    }
+    for (size_t j = 0; j < h->ops.size(); ++j) {
+        if (group[j].empty()) continue;
+        qx_ctx::Seg sg;
+        sg.level = h->ops[j].level;
+        sg.ops = group[j];
+        sg.plan = std::make_shared<SegPlan>(seg_plan(h, sg.ops, producer));
+        const SegPlan& p = *sg.plan;
+        if (p.arena > kSegArena[sg.level]) continue;
+        sg.wave = sg.level == 0;
+        for (auto& t : p.in) sg.wave = sg.wave && seg_storage(h, h->ops[sg.ops[t.op]], t.side) < 0;
+        if (!sg.wave && sg.ops.size() < 2) continue;
+        for (auto& t : p.in) {
+            const int sid = seg_storage(h, h->ops[sg.ops[t.op]], t.side);
+            if (sid >= 0) h->stor[sid].last = std::max(h->stor[sid].last, h->ops[j].step);
+        }
+        if (sg.wave) h->stor[h->ops[j].dst].def = 0;
+        for (int i : sg.ops) h->seg_of[i] = (int)h->segs.size();
+        h->segs.push_back(sg);
+    }
+}
+
+// The device programs of the segments (offsets are known)
+static void build_segments(qx_ctx* h) {
+    h->seg_blob.clear();
+    h->n_waves = 0;
+    h->wave_ok = false;
+    h->wave_flops = h->wave_bytes = 0;
+    h->chain_of_op.assign(h->ops.size(), -1);
+    std::vector<int32_t> wave_offs;
+    for (auto& sg : h->segs) {
+        const SegPlan& p = *sg.plan;
+        const int n = (int)sg.ops.size();
+        std::vector<SegIn> ins;
+        for (auto& t : p.in) {
+            const Op& op = h->ops[sg.ops[t.op]];
+            SegIn in{};
+            in.rank = t.bits;
+            in.arena = t.off;
+            in.once = t.once;
+            in.natural = 1;
+            const int sid = seg_storage(h, op, t.side);
+            if (sid >= 0) {
+                in.off = h->stor[sid].off;
+                in.space = h->stor[sid].level;
+            } else {
+                const Node& nd = h->nodes[op.type == OP_PERM ? op.src : t.side ? op.y : op.x];
+                in.off = nd.leaf_off;
+                in.space = SEG_LEAF;
+                for (int b = 0; b < in.rank; ++b) {
+                    in.pos[b] = (int8_t)nd.pos[in.rank - 1 - b];
+                    if (in.pos[b] != b) in.natural = 0;
+                }
+                in.n_fix = (int32_t)nd.fix.size();
+                for (int f = 0; f < in.n_fix; ++f) {
+                    in.fix_src[f] = nd.fix[f].first;
+                    in.fix_stride[f] = (int32_t)nd.fix[f].second;
+                }
+            }
+            ins.push_back(in);
+        }
+        std::vector<SegOp> sops(n);
+        struct Bits { int bits = 0; uint32_t xy[2 * kSegMaxBits] = {0}, d[2 * kSegMaxBits] = {0}; };
+        std::vector<Bits> ob(n);  // every output bit's offsets
+        sg.flops = sg.bytes = 0;
+        for (int i = 0; i < n; ++i) {
+            const Op& op = h->ops[sg.ops[i]];
+            SegOp& o = sops[i];
+            Bits& w = ob[i];
+            auto at = [&](int side) {
+                const int t = p.src[i][side];
+                return t < 0 ? 0 : t < n ? p.made[t].off : p.in[t - n].off;
+            };
+            o.x = at(0);
+            o.y = at(1);
+            o.dst = i + 1 < n ? p.made[i].off : -1;
+            sg.flops += op.flops;
+            sg.bytes += op_bytes(h, op, 1);
+            if (op.type == OP_GEMM) {
+                o.kind = op.mb + op.nb <= 4 && op.kb >= 8 ? SEGOP_DOT : SEGOP_MAC;
+                w.bits = op.mb + op.nb;
+                o.kb = op.kb;
+                for (int b = 0; b < op.nb; ++b) w.xy[b] = (uint32_t)(1u << (op.b_km ? op.kb + b : b)) << 16;
+                for (int b = 0; b < op.mb; ++b) w.xy[op.nb + b] = 1u << (op.a_km ? op.kb + b : b);
+                for (int b = 0; b < op.kb; ++b)
+                    o.k[b] = (1u << (op.a_km ? b : op.mb + b)) | ((uint32_t)(1u << (op.b_km ? b : op.nb + b)) << 16);
+            } else {
+                const Node& X = h->nodes[op.type == OP_PERM ? op.src : op.x];
+                const int rx = (int)X.legs.size();
+                auto pos = [](const Node& nd, int leg) {
+                    return (int)nd.legs.size() - 1 -
+                           (int)(std::find(nd.legs.begin(), nd.legs.end(), leg) - nd.legs.begin());
+                };
+                if (op.type == OP_PERM) {
+                    o.kind = SEGOP_COPY;
+                    w.bits = rx;
+                    for (int b = 0; b < rx; ++b) w.xy[b] = 1u << pos(X, op.target_legs[rx - 1 - b]);
+                } else {
+                    const Node& Y = h->nodes[op.y];
+                    o.kind = SEGOP_MAC;
+                    w.bits = op.mb + op.nb;
+                    o.kb = op.kb;
+                    for (int b = 0; b < op.nb; ++b) w.xy[b] = (uint32_t)(1u << pos(Y, op.fy[op.nb - 1 - b])) << 16;
+                    int m = op.nb;
+                    for (int j = rx - 1; j >= 0; --j)
+                        if (std::find(op.shared.begin(), op.shared.end(), X.legs[j]) == op.shared.end())
+                            w.xy[m++] = 1u << (rx - 1 - j);
+                    for (int b = 0; b < op.kb; ++b)
+                        o.k[b] = (1u << pos(X, op.shared[b])) | ((uint32_t)(1u << pos(Y, op.shared[b])) << 16);
+                }
+            }
+            for (int b = 0; b < w.bits; ++b) w.d[b] = 1u << (op.out_pos.empty() ? b : op.out_pos[b]);
+            for (int b = 0; b < std::min(w.bits, 5); ++b) {
+                o.xy[b] = w.xy[b];
+                o.d[b] = (uint16_t)w.d[b];
+            }
+        }
+        // tasks by stage: 32 outputs each (a dot product: one)
+        std::vector<SegTask> tasks;
+        std::vector<int32_t> bound;
+        sg.warp_clocks = 0;
+        for (int st = 0; st < p.n_stages; ++st) {
+            bound.push_back((int32_t)tasks.size());
+            for (int i = 0; i < n; ++i) {
+                if (p.stage[i] != st) continue;
+                const SegOp& o = sops[i];
+                const int outs = 1 << ob[i].bits, piece = o.kind == SEGOP_DOT ? 1 : std::min(outs, 32);
+                for (int o0 = 0; o0 < outs; o0 += piece) {
+                    SegTask t{i, piece, 0, 0};
+                    for (int b = 0; b < ob[i].bits; ++b)
+                        if ((o0 >> b) & 1) {
+                            t.xy += ob[i].xy[b];
+                            t.d += ob[i].d[b];
+                        }
+                    tasks.push_back(t);
+                }
+                sg.warp_clocks += (double)(outs / piece) * (70 + 9.0 * (1 << (o.kind == SEGOP_COPY ? 0 : o.kb)));
+            }
+        }
+        bound.push_back((int32_t)tasks.size());
+        SegHdr hd{};
+        hd.n_in = (int32_t)ins.size();
+        hd.n_ops = n;
+        hd.n_tasks = (int32_t)tasks.size();
+        hd.n_stages = p.n_stages;
+        hd.n_tiny = p.n_tiny;
+        hd.arena = p.arena;
+        const Storage& out = h->stor[h->ops[sg.ops.back()].dst];
+        hd.out_space = out.level;
+        hd.out_entries = (int32_t)out.entries;
+        hd.out_off = out.off;
+        sg.prog_off = (int64_t)h->seg_blob.size();
+        auto put = [&](const void* d, size_t bytes) {
+            const size_t at = h->seg_blob.size();
+            h->seg_blob.resize(at + (bytes + 15) / 16 * 16);
+            if (bytes) memcpy(h->seg_blob.data() + at, d, bytes);
+        };
+        put(&hd, sizeof hd);
+        put(ins.data(), ins.size() * sizeof(SegIn));
+        put(sops.data(), sops.size() * sizeof(SegOp));
+        put(tasks.data(), tasks.size() * sizeof(SegTask));
+        put(bound.data(), bound.size() * sizeof(int32_t));
+        sg.prog_bytes = (int32_t)((int64_t)h->seg_blob.size() - sg.prog_off);
+        ((SegHdr*)(h->seg_blob.data() + sg.prog_off))->bytes = sg.prog_bytes;
+        sg.arena = p.arena;
+        sg.n_stages = p.n_stages;
+        sg.n_tasks = (int)tasks.size();
+        if (sg.wave) {
+            for (int i : sg.ops) h->chain_of_op[i] = h->n_waves;
+            wave_offs.push_back((int32_t)sg.prog_off);
+            h->wave_flops += sg.flops;
+            h->wave_bytes += sg.bytes;
+            h->n_waves++;
+        }
+    }
+    h->wave_ok = h->n_waves > 0;
+    h->wave_list = (int64_t)h->seg_blob.size();
+    const uint8_t* w = (const uint8_t*)wave_offs.data();
+    h->seg_blob.insert(h->seg_blob.end(), w, w + wave_offs.size() * sizeof(int32_t));
+}
+
+// warps of a segment's CTA: many for a few items (latency), few when the items fill the GPU
+static int seg_threads(int64_t n_items) { return n_items >= 2048 ? 128 : n_items >= 512 ? 256 : 512; }
+
+// Whether running the segment beats a launch per step over n_items items.  A few items: the segment's
+// latency (a launch, its operands, 0.35 us a stage: 10 to 25 us measured) against the launches' (2.5 us
+// each, measured 3 to 5 and partly side by side).  Many items: the segment's issue time, 3.5 times its
+// estimated clocks (measured 189 and 420 us where 58 and 117 were estimated, on 16384 pairs: bank
+// conflicts of the strided reads), against the launches' bytes through HBM (62 and 133 us there).
+static bool seg_pays(const qx_ctx::Seg& sg, int64_t n_items) {
+    const double lat = 4.0 + 0.35 * sg.n_stages;
+    const double issue = 3.5 * (double)n_items * sg.warp_clocks / (152 * 4) / 1.9e3;
+    const double launches = std::max(2.5 * (double)sg.ops.size(), (double)n_items * sg.bytes / 4.5e6);
+    return std::max(lat, issue) < launches;
 }
 
 // how many distinct copies of a tensor of level `level` a launch of op over n_items items (n_b
@@ -1716,8 +2063,9 @@ struct Dag {
     std::vector<int> stream_of, last_on;  // per op: stream this batch (-1 none); per stream: last op
     std::vector<std::vector<int>> seen;   // seen[s][t]: latest op of stream t that stream s waited for
     std::vector<char> forked;
-    std::vector<int> wave_seen;          // per stream: 0 once it waited for the prologue launch
+    std::vector<char> wave_seen;         // per stream: it waited for the prologue launch
     bool waves_now = false;              // the prologue launch was issued in this batch
+    std::vector<char> seg_run;           // per segment: runs as one launch in this batch
     explicit Dag(qx_ctx* hh) : h(hh) {}
     int init() {
         on = h->n_streams > 1 && !h->profiling && !h->ops.empty();
@@ -1737,52 +2085,67 @@ struct Dag {
             CUDA_TRY(h, cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
             h->op_ev.push_back(e);
         }
-        while (h->wave_ok && h->wave_ev.empty()) {
-            cudaEvent_t e;
-            CUDA_TRY(h, cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-            h->wave_ev.push_back(e);
-        }
+        if (h->wave_ok && !h->wave_ev) CUDA_TRY(h, cudaEventCreateWithFlags(&h->wave_ev, cudaEventDisableTiming));
         return QX_OK;
     }
-    // the invariant steps, one launch on the handle's stream: one CTA per chain
-    int waves(const uint8_t* d_bits) {
+    SegCtx seg_ctx(const ItemCtx& ic, int64_t n_items, int level) const {
+        SegCtx c{};
+        c.leaves = (const float2*)(h->ws + h->off_leaf);
+        c.region[0] = inv_base(h);
+        c.region[1] = slice_base(h);
+        c.region[2] = item_base(h);
+        c.cap[0] = 1;
+        c.cap[1] = h->slices_cap;
+        c.cap[2] = h->items_cap;
+        c.n_items = n_items;
+        c.per_pair = level == 2;
+        c.ic = ic;
+        return c;
+    }
+    // the invariant segments that read only leaves, one launch on the handle's stream: one CTA each
+    int waves(const ItemCtx& ic) {
         if (!h->wave_ok) return QX_OK;
-        const size_t n = h->wave_ops.size(), nc = h->wave_start.size() - 1;
-        char* wbase = h->ws + h->off_wave;
-        const int32_t* idx = (const int32_t*)(wbase + align_up((int64_t)(n * sizeof(POp)), 256));
-        const int32_t* starts = idx + align_up((int64_t)(n * sizeof(int32_t)), 256) / (int64_t)sizeof(int32_t);
-        if (!h->waves_on_device) {
-            CUDA_TRY(h, cudaMemcpyAsync(wbase, h->wave_ops.data(), n * sizeof(POp), cudaMemcpyHostToDevice, h->stream));
-            CUDA_TRY(h, cudaMemcpyAsync((void*)idx, h->wave_idx.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice,
-                                        h->stream));
-            CUDA_TRY(h, cudaMemcpyAsync((void*)starts, h->wave_start.data(), (nc + 1) * sizeof(int32_t),
-                                        cudaMemcpyHostToDevice, h->stream));
-            CUDA_TRY(h, cudaStreamSynchronize(h->stream));
-            h->waves_on_device = true;
-        }
-        PProg prog{};
-        prog.ops = (const POp*)wbase;
-        prog.n_ops = (int32_t)n;
-        prog.n_qubits = h->nq;
-        prog.leaves = (const float2*)(h->ws + h->off_leaf);
-        prog.inv = inv_base(h);
-        prog.bits = d_bits;
-        prog.n_b = 1;
-        prog.scratch_override = inv_base(h);
+        SegCtx c = seg_ctx(ic, 1, 0);
+        c.prog = (const uint8_t*)(h->ws + h->off_wave);
+        c.prog_off = (const int32_t*)(c.prog + h->wave_list);
+        for (const auto& sg : h->segs)
+            if (sg.wave) {
+                c.prog_bytes = std::max(c.prog_bytes, sg.prog_bytes);
+                c.arena = std::max(c.arena, sg.arena);
+            }
         size_t slot;
-        cudaError_t e = prof_begin(h, QX_KERNEL_WAVE, h->wave_flops[0], h->wave_bytes[0], &slot);
-        if (e == cudaSuccess) e = launch_chains(prog.ops, idx, starts, (int)nc, prog, h->stream);
+        cudaError_t e = prof_begin(h, QX_KERNEL_WAVE, h->wave_flops, h->wave_bytes, &slot);
+        if (e == cudaSuccess) e = launch_seg(c, h->n_waves, 512, h->stream);
         if (e == cudaSuccess) e = prof_end(h, slot);
-        if (e == cudaSuccess && on) e = cudaEventRecord(h->wave_ev[0], h->stream);
+        if (e == cudaSuccess && on) e = cudaEventRecord(h->wave_ev, h->stream);
         if (e != cudaSuccess) return fail(h, QX_ECUDA, "prologue launch failed: %s", cudaGetErrorString(e));
         h->last_launches++;
-        h->last_flops += h->wave_flops[0];
+        h->last_flops += h->wave_flops;
         waves_now = true;
         if (on) last_on[0] = INT32_MAX / 2;  // per-pair steps go to the other streams first
         return QX_OK;
     }
+    int run_seg(const qx_ctx::Seg& sg, const ItemCtx& ic, int64_t n_items, cudaStream_t st) {
+        SegCtx c = seg_ctx(ic, n_items, sg.level);
+        c.prog = (const uint8_t*)(h->ws + h->off_wave) + sg.prog_off;
+        c.prog_bytes = sg.prog_bytes;
+        c.arena = sg.arena;
+        size_t slot;
+        cudaError_t e = prof_begin(h, QX_KERNEL_WAVE, sg.flops * (double)n_items, 0.0, &slot);
+        if (e == cudaSuccess) e = launch_seg(c, 1, seg_threads(n_items), st);
+        if (e == cudaSuccess) e = prof_end(h, slot);
+        if (e != cudaSuccess) return fail(h, QX_ECUDA, "segment launch failed: %s", cudaGetErrorString(e));
+        h->last_launches++;
+        h->last_flops += sg.flops * (double)n_items;
+        return QX_OK;
+    }
     cudaStream_t stream(int s) const { return s == 0 ? h->stream : h->dstreams[s - 1]; }
-    int fork() {
+    // n_items[level]: the items a step of that level runs over in this batch
+    int fork(const int64_t* n_items) {
+        seg_run.assign(h->segs.size(), 0);
+        for (size_t i = 0; i < h->segs.size(); ++i)
+            seg_run[i] = h->segs[i].wave || seg_pays(h->segs[i], n_items[h->segs[i].level]);
+        waves_now = false;
         if (!on) return QX_OK;
         const int S = h->n_streams;
         stream_of.assign(h->ops.size(), -1);
@@ -1790,21 +2153,35 @@ struct Dag {
         seen.assign(S, std::vector<int>(S, -1));
         forked.assign(S, 0);
         forked[0] = 1;
-        wave_seen.assign(S, -1);
-        waves_now = false;
+        wave_seen.assign(S, 0);
         CUDA_TRY(h, cudaEventRecord(h->fork_ev, h->stream));
         return QX_OK;
     }
     int issue(int j, const ItemCtx& ic, int64_t n_items) {
-        if (h->wave_ok && h->wave_of[j] >= 0) return QX_OK;  // ran in the prologue launch
-        if (!on) return run_op(h, h->ops[j], ic, n_items, h->stream);
-        const int S = h->n_streams;
-        int s = -1, wneed = -1;
-        for (int i : h->deps[j]) {
-            if (h->wave_ok && h->wave_of[i] >= 0) {
-                if (waves_now) wneed = std::max(wneed, h->wave_of[i]);
-                continue;
+        const int sid = h->seg_of[j] >= 0 && seg_run[h->seg_of[j]] ? h->seg_of[j] : -1;
+        const qx_ctx::Seg* sg = sid >= 0 ? &h->segs[sid] : nullptr;
+        if (sg && (sg->wave || sg->ops.back() != j)) return QX_OK;  // its segment's launch runs it
+        if (!on) return sg ? run_seg(*sg, ic, n_items, h->stream) : run_op(h, h->ops[j], ic, n_items, h->stream);
+        // the launches to follow: those of the op's dependencies (of all the segment's ops).  An op of
+        // a segment is run by the segment's last op; an inner op of a segment that comes later shares
+        // only its unused storage with this launch.
+        std::vector<int> after;
+        bool wneed = false;
+        auto follow = [&](int op) {
+            for (int i : h->deps[op]) {
+                const int t = h->seg_of[i] >= 0 && seg_run[h->seg_of[i]] ? h->seg_of[i] : -1;
+                if (t >= 0 && t == sid) continue;
+                if (t >= 0 && h->segs[t].wave) wneed = wneed || waves_now;
+                else after.push_back(t >= 0 ? h->segs[t].ops.back() : i);
             }
+        };
+        if (sg)
+            for (int op : sg->ops) follow(op);
+        else
+            follow(j);
+        const int S = h->n_streams;
+        int s = -1;
+        for (int i : after) {
             const int t = stream_of[i];
             if (t >= 0 && last_on[t] == i && (s < 0 || i > last_on[s])) s = t;
         }
@@ -1815,13 +2192,12 @@ struct Dag {
             CUDA_TRY(h, cudaStreamWaitEvent(stream(s), h->fork_ev, 0));
             forked[s] = 1;
         }
-        if (wneed >= 0 && s != 0 && wave_seen[s] < wneed) {
-            CUDA_TRY(h, cudaStreamWaitEvent(stream(s), h->wave_ev[wneed], 0));
-            wave_seen[s] = wneed;
+        if (wneed && s != 0 && !wave_seen[s]) {
+            CUDA_TRY(h, cudaStreamWaitEvent(stream(s), h->wave_ev, 0));
+            wave_seen[s] = 1;
         }
         std::vector<int> latest(S, -1);
-        for (int i : h->deps[j]) {
-            if (h->wave_ok && h->wave_of[i] >= 0) continue;
+        for (int i : after) {
             const int t = stream_of[i];
             if (t >= 0 && t != s) latest[t] = std::max(latest[t], i);
         }
@@ -1830,7 +2206,7 @@ struct Dag {
                 CUDA_TRY(h, cudaStreamWaitEvent(stream(s), h->op_ev[latest[t]], 0));
                 seen[s][t] = latest[t];
             }
-        int rc = run_op(h, h->ops[j], ic, n_items, stream(s));
+        int rc = sg ? run_seg(*sg, ic, n_items, stream(s)) : run_op(h, h->ops[j], ic, n_items, stream(s));
         if (rc) return rc;
         CUDA_TRY(h, cudaEventRecord(h->op_ev[j], stream(s)));
         stream_of[j] = s;
@@ -1860,6 +2236,12 @@ static int contract_impl(qx_ctx* h, const uint8_t* d_bits, int64_t n_bits, int64
                                     cudaMemcpyHostToDevice, h->stream));
         CUDA_TRY(h, cudaStreamSynchronize(h->stream));
         h->leaves_on_device = true;
+    }
+    if (!h->segs_on_device && !h->seg_blob.empty()) {
+        CUDA_TRY(h, cudaMemcpyAsync(h->ws + h->off_wave, h->seg_blob.data(), h->seg_blob.size(),
+                                    cudaMemcpyHostToDevice, h->stream));
+        CUDA_TRY(h, cudaStreamSynchronize(h->stream));
+        h->segs_on_device = true;
     }
     double* acc = (double*)(h->ws + h->off_acc);
     CUDA_TRY(h, cudaMemsetAsync(h->ws + h->off_err, 0, sizeof(int), h->stream));
@@ -1918,8 +2300,9 @@ static int contract_impl(qx_ctx* h, const uint8_t* d_bits, int64_t n_bits, int64
             ic.b0 = b0;
             ic.n_b = (int32_t)nb;
             ic.n_items = ns * nb;
-            if ((rc = dag.fork())) return rc;
-            if (prologue && (rc = dag.waves(d_bits))) return rc;
+            const int64_t level_items[3] = {1, ns, ns * nb};
+            if ((rc = dag.fork(level_items))) return rc;
+            if (prologue && (rc = dag.waves(ic_inv))) return rc;
             ItemCtx ic_s = ic;
             ic_s.n_b = 1;
             ic_s.n_items = ns;
@@ -2042,7 +2425,7 @@ void qx_destroy(qx_handle h) {
     for (cudaEvent_t e : h->ev_pool) cudaEventDestroy(e);
     for (cudaEvent_t e : h->op_ev) cudaEventDestroy(e);
     for (cudaEvent_t e : h->join_ev) cudaEventDestroy(e);
-    for (cudaEvent_t e : h->wave_ev) cudaEventDestroy(e);
+    if (h->wave_ev) cudaEventDestroy(h->wave_ev);
     for (auto& kv : h->reqs) cudaEventDestroy(kv.second);
     for (cudaEvent_t e : h->req_pool) cudaEventDestroy(e);
     if (h->fork_ev) cudaEventDestroy(h->fork_ev);
@@ -2101,7 +2484,7 @@ static void unbind(qx_ctx* h) {
     h->items_cap = 0;
     h->leaves_on_device = false;
     h->pops_on_device = false;
-    h->waves_on_device = false;
+    h->segs_on_device = false;
     h->inv_ready = false;
 }
 
@@ -2138,8 +2521,7 @@ int qx_bind_workspace(qx_handle h, void* dptr, int64_t bytes, int64_t max_bits) 
     if (((uintptr_t)dptr) % 256) return fail(h, QX_EINVAL, "workspace must be 256-byte aligned");
     unbind(h);
     int64_t fixed, items = 0, slices = 0;
-    layout(h, max_bits, &fixed);
-    if (!fit_regions(h, bytes - fixed, max_bits, &items, &slices))
+    if (!fit_layout(h, bytes, nullptr, max_bits, &fixed, &items, &slices))
         return fail(h, QX_ENOMEM, "workspace of %lld bytes holds no (slice, bitstring) pair; need %lld", (long long)bytes,
                     (long long)(fixed + 256 + (h->item_entries + h->slice_entries) * 8));
     CUDA_TRY(h, cudaSetDevice(h->device));
@@ -2153,7 +2535,7 @@ int qx_bind_workspace(qx_handle h, void* dptr, int64_t bytes, int64_t max_bits) 
     place_regions(h, fixed, items, slices);
     h->leaves_on_device = false;
     h->pops_on_device = false;
-    h->waves_on_device = false;
+    h->segs_on_device = false;
     return QX_OK;
 }
 
@@ -2183,10 +2565,10 @@ int qx_bind_workspace_parts(qx_handle h, void* d_fixed, int64_t fixed_bytes, voi
         return fail(h, QX_EINVAL, "a split workspace is for the batched executor");
     unbind(h);
     int64_t fixed, items = 0, slices = 0;
-    layout(h, max_bits, &fixed);
+    const bool fits = fit_layout(h, fixed_bytes, &batch_bytes, max_bits, &fixed, &items, &slices);
     if (fixed_bytes < fixed)
         return fail(h, QX_ENOMEM, "fixed part of %lld bytes; need %lld", (long long)fixed_bytes, (long long)fixed);
-    if (!fit_regions(h, batch_bytes, max_bits, &items, &slices))
+    if (!fits)
         return fail(h, QX_ENOMEM, "batch part of %lld bytes holds no (slice, bitstring) pair; need %lld",
                     (long long)batch_bytes, (long long)(256 + (h->item_entries + h->slice_entries) * 8));
     h->ws = (char*)d_fixed;
@@ -2196,7 +2578,7 @@ int qx_bind_workspace_parts(qx_handle h, void* d_fixed, int64_t fixed_bytes, voi
     place_regions(h, 0, items, slices);
     h->leaves_on_device = false;
     h->pops_on_device = false;
-    h->waves_on_device = false;
+    h->segs_on_device = false;
     return QX_OK;
 }
 
@@ -2428,6 +2810,10 @@ int qx_describe_plan(qx_handle h, char* buf, int64_t len, int64_t* needed) {
             snprintf(line, sizeof line, " chain=%d", h->chain_of_op[i]);
             out += line;
         }
+        else if (h->seg_of[i] >= 0) {  // one launch with the other steps of this segment when that pays
+            snprintf(line, sizeof line, " seg=%d", h->seg_of[i]);
+            out += line;
+        }
         out += "\n";
     }
     if (needed) *needed = (int64_t)out.size() + 1;
@@ -2556,15 +2942,16 @@ int qx_internal_contract_in(qx_ctx* h, char* buf, int64_t buf_bytes, const uint8
             slices_cap;
         bool leaves_on_device;
         int64_t off_pops, off_counter, off_results, off_pscratch, off_pops_inv, off_wave;
-        bool pops_on_device, waves_on_device, inv_ready;
+        bool pops_on_device, segs_on_device, inv_ready;
     } const saved = {h->ws,        h->ws_bytes, h->ws_owned,    h->max_bits,    h->off_err,    h->off_leaf,
                      h->off_bits,  h->off_acc,  h->off_amps,    h->off_inv,     h->off_item,   h->items_cap,
                      h->off_slice, h->slices_cap, h->leaves_on_device, h->off_pops, h->off_counter, h->off_results, h->off_pscratch,
-                     h->off_pops_inv, h->off_wave, h->pops_on_device, h->waves_on_device, h->inv_ready};
+                     h->off_pops_inv, h->off_wave, h->pops_on_device, h->segs_on_device, h->inv_ready};
     int64_t fixed, items = 0, slices = 0;
-    layout(h, n_bits, &fixed);
-    const bool fits = fit_regions(h, buf_bytes - fixed, n_bits, &items, &slices);
+    const bool saved_segs = h->segs_on;
+    const bool fits = fit_layout(h, buf_bytes, nullptr, n_bits, &fixed, &items, &slices);
     auto restore = [&]() {
+        if (h->segs_on != saved_segs) finish_layout(h, saved_segs);  // the bound workspace's layout
         h->ws = saved.ws;
         h->ws_bytes = saved.ws_bytes;
         h->ws_owned = saved.ws_owned;
@@ -2587,7 +2974,7 @@ int qx_internal_contract_in(qx_ctx* h, char* buf, int64_t buf_bytes, const uint8
         h->off_pops_inv = saved.off_pops_inv;
         h->pops_on_device = saved.pops_on_device;
         h->off_wave = saved.off_wave;
-        h->waves_on_device = saved.waves_on_device;
+        h->segs_on_device = saved.segs_on_device;
         h->inv_ready = saved.inv_ready;
     };
     if (!fits) {
@@ -2605,7 +2992,7 @@ int qx_internal_contract_in(qx_ctx* h, char* buf, int64_t buf_bytes, const uint8
     place_regions(h, fixed, items, slices);
     h->leaves_on_device = false;
     h->pops_on_device = false;
-    h->waves_on_device = false;
+    h->segs_on_device = false;
     h->inv_ready = false;  // the shared scratch array holds whatever the last call left
     int rc = QX_OK;
     cudaError_t e = cudaSetDevice(h->device);

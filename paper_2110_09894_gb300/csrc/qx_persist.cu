@@ -386,39 +386,6 @@ cudaError_t launch_group_sum(const GSum* d_sums, int32_t n, int64_t total, cudaS
     return cudaGetLastError();
 }
 
-// ---- the invariant steps in one launch -----------------------------------------------------------
-// The steps that no slice or bitstring touches are mostly tiny (gate-sized tensors).  The plan
-// compiler splits them into chains that share no storage (their dependency trees, with the
-// invariant region given no reuse): CTA c runs the steps of chain c in plan order with the code of
-// the persistent executor, a block barrier between steps, and waits for no other CTA.
-__global__ void __launch_bounds__(256, 2) k_chain(const POp* __restrict__ ops, const int32_t* __restrict__ idx,
-                                                  const int32_t* __restrict__ starts, const PProg prog) {
-    extern __shared__ float2 psm[];
-    PairCtx c;
-    c.s = 0;
-    c.bits = prog.bits;
-    c.scratch = prog.scratch_override;
-    c.prog = &prog;
-    const int i1 = starts[blockIdx.x + 1];
-    for (int i = starts[blockIdx.x]; i < i1; ++i) {
-        const POp& op = ops[idx[i]];
-        switch (op.type) {
-            case POP_PERM: exec_perm(op, c, psm); break;
-            case POP_SMALL: exec_small(op, c, psm); break;
-            case POP_GEMM: exec_gemm(op, c, psm); break;
-            default: exec_dot(op, c, psm); break;
-        }
-        __syncthreads();  // this step's results (global and shared) before the next step reads them
-    }
-}
-
-cudaError_t launch_chains(const POp* ops, const int32_t* idx, const int32_t* starts, int n_chains, const PProg& prog,
-                          cudaStream_t st) {
-    if (n_chains <= 0) return cudaSuccess;
-    k_chain<<<n_chains, 256, kPersistSmem, st>>>(ops, idx, starts, prog);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_persist(const PLaunch& L, int grid, cudaStream_t st) {
     if (L.n_work <= 0) return cudaSuccess;
     cudaError_t e = cudaMemsetAsync(L.counter, 0, sizeof(unsigned long long), st);
