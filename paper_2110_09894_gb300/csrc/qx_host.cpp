@@ -1439,11 +1439,15 @@ static double op_bytes(const qx_ctx* h, const Op& op, int64_t n_items, int64_t n
 // Segments: connected groups of small steps of one level, run by one launch (qx_seg.cu)
 // ------------------------------------------------------------------------------------------------
 constexpr int kSegOps = 200;               // steps of one segment
+constexpr int64_t kSegTasks = 2048;        // its 32-output pieces (16 bytes each in its program)
 constexpr int64_t kSegArena[3] = {12288, 4096, 4096};  // arena entries by level (8 bytes each)
 constexpr int kSegBits[3] = {12, 10, 10};  // largest tensor
 constexpr int kSegMacs[3] = {17, 14, 14};  // largest step, log2 of M K N
 
 // operand `side` (0: X / A, 1: Y / B) of an op: its node (gathers, permutes) or storage (GEMM), -1 if none
+static_assert(kSegOps * (int)sizeof(SegOp) + (kSegOps + 1) * (int)sizeof(SegIn) + kSegTasks * (int)sizeof(SegTask) +
+                      (kSegOps + 1) * 4 + (int)sizeof(SegHdr) + 80 + kSegArena[0] * 8 <= kSegMaxSmem,
+              "a segment's program and arena fit in shared memory");
 static int seg_storage(const qx_ctx* h, const Op& op, int side) {
     if (op.type == OP_GEMM) return side ? op.sb : op.sa;
     const int node = op.type == OP_PERM ? (side ? -1 : op.src) : side ? op.y : op.x;
@@ -1585,10 +1589,13 @@ static void choose_segments(qx_ctx* h) {
     const std::vector<int> producer = storage_producers(h);
     std::vector<std::vector<int>> group(h->ops.size());  // by root op, plan order
     std::vector<int64_t> flat(h->ops.size(), 0);         // entries of all its steps' operands and results
+    std::vector<int64_t> pieces(h->ops.size(), 0);       // tasks of its steps
     for (size_t j = 0; j < h->ops.size(); ++j) {
         const Op& op = h->ops[j];
         if (!seg_able(h, op)) continue;
         group[j] = {(int)j};
+        pieces[j] = op.type == OP_GEMM && op.mb + op.nb <= 4 && op.kb >= 8 ? h->stor[op.dst].entries
+                                                                           : std::max<int64_t>(1, h->stor[op.dst].entries / 32);
         flat[j] = std::max<int64_t>(2, h->stor[op.dst].entries);
         for (int side = 0; side < 2; ++side) flat[j] += std::max(2, 1 << seg_operand_bits(h, op, side));
         for (int side = 0; side < 2; ++side) {
@@ -1600,10 +1607,11 @@ static void choose_segments(qx_ctx* h) {
             std::sort(both.begin(), both.end());
             // the arena of everything at once bounds the one of the stages
             const int64_t all = flat[i] + flat[j];
-            if ((int)both.size() > kSegOps ||
+            if ((int)both.size() > kSegOps || pieces[i] + pieces[j] > kSegTasks ||
                 (all > kSegArena[op.level] && seg_plan(h, both, producer).arena > kSegArena[op.level]))
                 continue;
             flat[j] = all;
+            pieces[j] += pieces[i];
             group[j] = both;
             group[i].clear();
         }

@@ -61,3 +61,31 @@ def test_a_workspace_too_small_for_segments_still_contracts(qx, no_slice_level):
         assert np.array_equal(s.contract(bits), want)
         s.close()
     assert fitted and not fitted[0]  # the smaller layout fits a little below the segments' need
+
+
+def test_a_long_run_of_large_steps_is_cut_into_segments_that_fit(qx):
+    """A chain of dozens of steps on 2^12-entry tensors: each has 128 pieces of work, so a segment of all
+    of them would not fit in shared memory."""
+    n = 12
+    circ = C.Circuit(n)
+    rng = C.SplitMix64(9)
+    for t in range(6):
+        for q in range(n):
+            circ.append((q,), C.ONE_QUBIT_SET[rng.randint(3)])
+        for q in range(t % 2, n - 1, 2):
+            circ.append((q, q + 1), C.FSIM_SYC)
+    om = np.ones(n, np.uint8)
+    om[0] = 0
+    recs = C.gates_to_records(circ)
+    # state-vector order: the inputs joined first, then every gate onto the state
+    order, cur = [], 0
+    total = n + len(circ.gates) + 1
+    for t in list(range(1, n + len(circ.gates) + 1)):
+        order.append((cur, t))
+        cur = total + len(order) - 1
+    c = qx.Contractor(n, recs, om, order, [], 2)
+    bits = np.zeros((2, n), np.uint8)
+    bits[1, 0] = 1
+    got = c.contract(bits)
+    c.close()
+    assert_parity(got, oracle.sv_amplitudes(n, recs, om, bits))
