@@ -612,7 +612,7 @@ constexpr int GBK = 16;
 constexpr int GFOLD = 4;  // stages per partial
 
 template <int BM, int BN>
-__global__ void __launch_bounds__(256, (BM * BN >= 8192 ? 1 : 2)) k_gemm_c64(const float2* __restrict__ A, int64_t a_is, bool akm,
+__global__ void __launch_bounds__(256, 2) k_gemm_c64(const float2* __restrict__ A, int64_t a_is, bool akm,
                                                   const float2* __restrict__ B, int64_t b_is, bool bkm,
                                                   float2* __restrict__ C, int64_t c_is, int mb, int nb, int kb,
                                                   int tiles_n, const __grid_constant__ OutMap om, int a_div,
@@ -733,6 +733,177 @@ __global__ void __launch_bounds__(256, (BM * BN >= 8192 ? 1 : 2)) k_gemm_c64(con
             if (gn < N) Cp[gm * N + gn] = tot[i][j];
         }
     }
+}
+
+// ---------------------------------------------------------------------------------------------
+// The same GEMM on packed FP32 FMAs (fma.rn.f32x2), for M, N >= 32 and K >= 8.  An FMA with three
+// different register operands issues at 0.7 of the FP32 rate here (57 of 80 TFLOP/s in a register-only
+// loop; packed 64), and a complex multiply-add takes four, so k_gemm_c64 filled its issue slots (80%,
+// FMA pipe 56%) at 30 to 47 TFLOP/s.  Packed, a multiply-add is two instructions on (re, im) sums,
+//     acc += (ar, ar) * (br, bi),   acc += (ai, ai) * (-bi, br),
+// the same four roundings in the same order.  The operands stay 8 bytes in shared memory and are
+// doubled in registers: reading them doubled (16 bytes) costs 48 clocks of the load path per k and
+// warp against 32 to 40 of the FMAs (measured: 38 to 47 TFLOP/s).  64 x 64 outputs (32 on a short
+// side) per CTA, 8 x 4 per thread, 8 k per stage, register-staged double buffer; 64 x 64 rather than
+// 128 x 64 so that several CTAs per SM cover each other's barriers.  FOLD (K > 64): sums of 64 k are
+// added to running totals (see above), kept in shared memory so that the registers hold three CTAs
+// per SM; shorter sums need no total.  Now bound by the packed FMAs' operand reads (pipe 67% busy).
+// Before / after (us): 64 x 128 x 64 for 16384 items 1571 / 1420; 32 x 256 x 64 for 16384 1898 / 1428;
+// 2048 x 512 x 512 for 64 5897 / 5409; 2^15 x 32 x 32 for 64 545 / 371; 256 x 512 x 8 for 1024 455 / 261.
+// ---------------------------------------------------------------------------------------------
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
+    unsigned long long d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
+__device__ __forceinline__ unsigned long long pair2(float lo, float hi) {
+    unsigned long long d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
+    return d;
+}
+
+constexpr int PBK = 8;  // k per stage
+template <int BM, int BN, bool FOLD>
+struct PackedTile {
+    static constexpr int NT = BM * BN / 32;                       // threads
+    static constexpr int RA = BM * PBK / NT, RB = BN * PBK / NT;  // entries per thread and stage
+    static constexpr int SMEM = 8 * (2 * PBK * (BM + 1 + BN + 1) + (FOLD ? BM * BN : 0));
+};
+
+template <int BM, int BN, bool FOLD>
+__global__ void __launch_bounds__(PackedTile<BM, BN, FOLD>::NT, (FOLD ? 384 : 512) / PackedTile<BM, BN, FOLD>::NT)
+    k_gemm_packed(const float2* __restrict__ A, int64_t a_is, bool akm, const float2* __restrict__ B, int64_t b_is,
+                  bool bkm, float2* __restrict__ C, int64_t c_is, int mb, int nb, int kb, int tiles_n,
+                  const __grid_constant__ OutMap om, int a_div, int b_div) {
+    using T = PackedTile<BM, BN, FOLD>;
+    constexpr int NT = T::NT, RA = T::RA, RB = T::RB, TX = BN / 4, TY = BM / 8;
+    extern __shared__ float2 gsm[];
+    float2(*As)[PBK][BM + 1] = (float2(*)[PBK][BM + 1])gsm;
+    float2(*Bs)[PBK][BN + 1] = (float2(*)[PBK][BN + 1])(gsm + 2 * PBK * (BM + 1));
+    unsigned long long* tot = (unsigned long long*)(gsm + 2 * PBK * (BM + 1 + BN + 1)) + threadIdx.x;  // [32][NT]
+    const int64_t M = (int64_t)1 << mb, N = (int64_t)1 << nb, K = (int64_t)1 << kb;
+    const int64_t item = blockIdx.y;
+    const int64_t m0 = (int64_t)(blockIdx.x / tiles_n) * BM;
+    const int64_t n0 = (int64_t)(blockIdx.x % tiles_n) * BN;
+    const int tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
+    // this thread's entries of a stage: K-major operands run along k, the others along their rows
+    const int a_k = akm ? tid % PBK : tid / BM, a_r = akm ? tid / PBK : tid % BM;
+    const int b_k = bkm ? tid % PBK : tid / BN, b_r = bkm ? tid / PBK : tid % BN;
+    const float2* Ap = A + (item / a_div) * a_is + (akm ? (m0 + a_r) * K + a_k : a_k * M + m0 + a_r);
+    const float2* Bp = B + (item / b_div) * b_is + (bkm ? (n0 + b_r) * K + b_k : b_k * N + n0 + b_r);
+    const int64_t a_step = akm ? (NT / PBK) * K : (NT / BM) * M, b_step = bkm ? (NT / PBK) * K : (NT / BN) * N;
+    const int64_t a_next = akm ? PBK : PBK * M, b_next = bkm ? PBK : PBK * N;
+    const int a_sk = akm ? 0 : NT / BM, a_sr = akm ? NT / PBK : 0, b_sk = bkm ? 0 : NT / BN, b_sr = bkm ? NT / PBK : 0;
+    float2 ra[RA], rb[RB];
+    auto gload = [&]() {
+#pragma unroll
+        for (int r = 0; r < RA; ++r) ra[r] = Ap[r * a_step];
+#pragma unroll
+        for (int r = 0; r < RB; ++r) rb[r] = Bp[r * b_step];
+        Ap += a_next;
+        Bp += b_next;
+    };
+    auto sstore = [&](int buf) {
+#pragma unroll
+        for (int r = 0; r < RA; ++r) As[buf][a_k + r * a_sk][a_r + r * a_sr] = ra[r];
+#pragma unroll
+        for (int r = 0; r < RB; ++r) Bs[buf][b_k + r * b_sk][b_r + r * b_sr] = rb[r];
+    };
+    unsigned long long acc[8][4];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = 0;
+    gload();
+    sstore(0);
+    __syncthreads();
+    const int stages = (int)(K / PBK);
+    for (int st = 0; st < stages; ++st) {
+        const int buf = st & 1;
+        const bool more = st + 1 < stages;
+        if (more) gload();
+#pragma unroll
+        for (int k = 0; k < PBK; ++k) {
+            unsigned long long b[4], bs[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float2 v = Bs[buf][k][tx + TX * j];
+                b[j] = pair2(v.x, v.y);
+                bs[j] = pair2(-v.y, v.x);
+            }
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const float2 v = As[buf][k][ty + TY * i];
+                const unsigned long long ar = pair2(v.x, v.x), ai = pair2(v.y, v.y);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[i][j] = fma2(ar, b[j], acc[i][j]);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[i][j] = fma2(ai, bs[j], acc[i][j]);
+            }
+        }
+        if (FOLD && (st & 7) == 7) {  // 64 k summed: into the totals, the first time as they are (0 + x)
+            const bool first = st == 7;
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const unsigned long long t = first ? acc[i][j] : add2(tot[(4 * i + j) * NT], acc[i][j]);
+                    if (more) {
+                        tot[(4 * i + j) * NT] = t;
+                        acc[i][j] = 0;
+                    } else {
+                        acc[i][j] = t;
+                    }
+                }
+        }
+        if (more) sstore(buf ^ 1);
+        __syncthreads();
+    }
+    float2* Cp = C + item * c_is;
+    int64_t co[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) co[j] = om.on ? place_bits(n0 + tx + TX * j, om.pos) : n0 + tx + TX * j;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int64_t gm = m0 + ty + TY * i;
+        const int64_t ro = om.on ? place_bits(gm, om.pos + nb) : gm * N;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) *(unsigned long long*)(Cp + ro + co[j]) = acc[i][j];
+    }
+}
+
+template <int BM, int BN, bool FOLD>
+static cudaError_t gemm_packed(cudaStream_t st, const float2* a, int64_t a_is, bool akm, const float2* b, int64_t b_is,
+                               bool bkm, float2* c, int64_t c_is, int mb, int nb, int kb, int64_t n_items,
+                               const OutMap& om, int a_div, int b_div) {
+    using T = PackedTile<BM, BN, FOLD>;
+    static_assert(T::NT % BM == 0 && T::NT % BN == 0 && T::NT % PBK == 0, "tile");
+    static_assert(T::SMEM <= 50 * 1024, "smem");
+    if (T::SMEM > 48 * 1024) {
+        // opt in to more than 48 KB of dynamic shared memory, once per device
+        static uint64_t done[4] = {};
+        static std::mutex mu;
+        int dev = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e != cudaSuccess) return e;
+        std::lock_guard<std::mutex> lk(mu);
+        if (dev >= 256 || !((done[dev >> 6] >> (dev & 63)) & 1)) {
+            e = cudaFuncSetAttribute(k_gemm_packed<BM, BN, FOLD>, cudaFuncAttributeMaxDynamicSharedMemorySize, T::SMEM);
+            if (e != cudaSuccess) return e;
+            if (dev < 256) done[dev >> 6] |= 1ull << (dev & 63);
+        }
+    }
+    const int64_t tm = (1ll << mb) / BM, tn = (1ll << nb) / BN;
+    const dim3 grid((unsigned)(tm * tn), (unsigned)n_items);
+    k_gemm_packed<BM, BN, FOLD><<<grid, T::NT, T::SMEM, st>>>(a, a_is, akm, b, b_is, bkm, c, c_is, mb, nb, kb, (int)tn,
+                                                              om, a_div, b_div);
+    return cudaGetLastError();
 }
 
 // Long dot products (M * N <= 16 outputs, large K): one CTA per item, the 256
@@ -938,7 +1109,23 @@ cudaError_t launch_gemm_c64(const float2* a, int64_t a_is, bool a_kmajor, const 
 #undef QX_DOT_CASE
         return cudaErrorInvalidValue;
     }
-    const int bmb = mb >= 7 && nb >= 6 ? 7 : mb >= 6 ? 6 : mb >= 5 ? 5 : 4;  // tile edge 128 / 64 / 32 / 16
+    if (mb >= 5 && nb >= 5 && kb >= 3) {
+#define QX_PACKED(X, Y)                                                                                             \
+    (kb > 6 ? gemm_packed<X, Y, true>(st, a, a_is, a_kmajor, b, b_is, b_kmajor, c, c_is, mb, nb, kb, n_items, om,  \
+                                      a_div, b_div)                                                                \
+            : gemm_packed<X, Y, false>(st, a, a_is, a_kmajor, b, b_is, b_kmajor, c, c_is, mb, nb, kb, n_items, om, \
+                                       a_div, b_div))
+        // the narrow tiles are CTAs of one or two warps: below 512 of them the 256-thread tiles of
+        // k_gemm_c64 are faster (300 products of 32 x 32 x 128: 12.8 us against 22.6; 512 tiles of 32 x 64
+        // x 128: 37.6 against 33.3)
+        if (mb > 5 && nb > 5) return QX_PACKED(64, 64);
+        if ((((1ll << mb) / (mb == 5 ? 32 : 64)) * ((1ll << nb) / (nb == 5 ? 32 : 64))) * n_items >= 512) {
+            if (nb == 5) return mb == 5 ? QX_PACKED(32, 32) : QX_PACKED(64, 32);
+            return QX_PACKED(32, 64);
+        }
+#undef QX_PACKED
+    }
+    const int bmb = mb >= 6 ? 6 : mb >= 5 ? 5 : 4;  // tile edge 64 / 32 / 16
     const int bnb = nb >= 6 ? 6 : nb >= 5 ? 5 : 4;
     const int64_t tm = ((1ll << mb) + (1 << bmb) - 1) >> bmb, tn = ((1ll << nb) + (1 << bnb) - 1) >> bnb;
     dim3 grid((unsigned)(tm * tn), (unsigned)n_items);
@@ -948,8 +1135,7 @@ cudaError_t launch_gemm_c64(const float2* a, int64_t a_is, bool a_kmajor, const 
                                       (int)tn, om, a_div, b_div);                                     \
         return cudaGetLastError();                                                                    \
     }
-    QX_GEMM_CASE(7, 6)
-    QX_GEMM_CASE(6, 6) QX_GEMM_CASE(6, 5) QX_GEMM_CASE(6, 4)
+    QX_GEMM_CASE(6, 5) QX_GEMM_CASE(6, 4)
     QX_GEMM_CASE(5, 6) QX_GEMM_CASE(5, 5) QX_GEMM_CASE(5, 4)
     QX_GEMM_CASE(4, 6) QX_GEMM_CASE(4, 5) QX_GEMM_CASE(4, 4)
 #undef QX_GEMM_CASE
