@@ -906,6 +906,165 @@ static cudaError_t gemm_packed(cudaStream_t st, const float2* a, int64_t a_is, b
     return cudaGetLastError();
 }
 
+// ---------------------------------------------------------------------------------------------
+// Products with a short side (at most 16 rows or columns): the work is reading the long operand, and a
+// 16-wide tile leaves most of a CTA idle (4 x 4 outputs over K = 64: 1/16 of its threads).  Here a CTA
+// of 256 threads takes `items` whole items or `lr` long rows of one, stages 64 G k of both operands in
+// shared memory with coalesced loads (rows padded to an odd stride), and each thread sums one output
+// over one 64-k chunk; G chunks of an output are summed side by side and then added in order, which
+// is the blocked sum of k_gemm_c64 (K <= 64: one chunk, no addition).  SWAP: A is the short operand.
+// Measured against the 16-wide tiles: 4 x 4 x 64 for 16384 items 119 -> 21 us; 4096 x 2 x 64 for 376 items
+// 457 -> 233 us; 16 x 4 x 4096 for 376 items 219 -> 135 us.  With 8 or 16 short rows the tiles are full
+// enough (256 x 16 x 64 for 4096 items 329 us, here 926), except for a few items of a long K, where the
+// tiles leave SMs idle and the chunks side by side win (4096 x 16 x 512, one item: 31 -> 25 us; 8 x 8 x
+// 512 for 96: 20.6 -> 10.3), and for both sides short (8 x 8 x 16 for 16384: 50 -> 33).
+// ---------------------------------------------------------------------------------------------
+constexpr int kSkinnySmem = 72 * 1024, kSkinnyMax = 4;
+struct SkinnyShape {   // log2 of everything
+    int lb, sb, kb;     // the long side, the short side, K
+    int lr, items, g;   // long rows per CTA, items per CTA (0 unless lr is the whole long side), chunks at a time
+    int kw;             // k per chunk: min(K, 64)
+};
+// rows 0 .. 2^rb - 1 (of row length 2^kb when K-major, of column length 2^colb else), k0 .. + 2^kt - 1, of
+// items item0 .. + np - 1 into dst[item][row][2^kt + 1]; two entries per load
+__device__ __forceinline__ void skinny_stage(float2* dst, const float2* __restrict__ src, int64_t is, int div,
+                                             int64_t item0, int np, bool kmaj, int rb, int kb, int colb, int64_t r0,
+                                             int k0, int kt) {
+    const int ld = (1 << kt) + 1, n = np << (rb + kt - 1);
+#pragma unroll 8
+    for (int i = threadIdx.x; i < n; i += 256) {
+        const int q = i >> (rb + kt - 1), e = i & ((1 << (rb + kt - 1)) - 1);
+        const float2* s = src + (int64_t)(uint32_t)((uint32_t)(item0 + q) / (uint32_t)div) * is;
+        if (kmaj) {
+            const int k = (e & ((1 << (kt - 1)) - 1)) * 2, r = e >> (kt - 1);
+            const float4 v = *(const float4*)(s + ((r0 + r) << kb) + k0 + k);
+            float2* d = dst + ((q << rb) + r) * ld + k;
+            d[0] = make_float2(v.x, v.y);
+            d[1] = make_float2(v.z, v.w);
+        } else if (rb > 0) {
+            const int r = (e & ((1 << (rb - 1)) - 1)) * 2, k = e >> (rb - 1);
+            const float4 v = *(const float4*)(s + ((int64_t)(k0 + k) << colb) + r0 + r);
+            float2* d = dst + ((q << rb) + r) * ld + k;
+            d[0] = make_float2(v.x, v.y);
+            d[ld] = make_float2(v.z, v.w);
+        } else {
+            for (int h = 0; h < 2; ++h) dst[q * ld + 2 * e + h] = s[((int64_t)(k0 + 2 * e + h) << colb) + r0];
+        }
+    }
+}
+template <bool SWAP>
+__global__ void __launch_bounds__(256) k_gemm_skinny(const float2* __restrict__ A, int64_t a_is, bool akm,
+                                                     const float2* __restrict__ B, int64_t b_is, bool bkm,
+                                                     float2* __restrict__ C, int64_t c_is, const SkinnyShape sh,
+                                                     const __grid_constant__ OutMap om, int a_div, int b_div,
+                                                     int64_t n_items) {
+    extern __shared__ float2 gsm[];
+    const int K = 1 << sh.kb, kt = sh.g + sh.kw, ld = (1 << kt) + 1, G = 1 << sh.g;
+    const int lr = 1 << sh.lr, P = 1 << sh.items, S = 1 << sh.sb;
+    float2* ls = gsm;                    // [P][lr][ld]
+    float2* ss = ls + P * lr * ld;       // [P][S][ld]
+    float2* red = ss + P * S * ld;       // [g][P][S][lr], g > 1
+    const int64_t item0 = (int64_t)blockIdx.y * P;
+    const int l0 = blockIdx.x * lr;
+    const int np = n_items - item0 < P ? (int)(n_items - item0) : P;
+    const int tid = threadIdx.x;
+    // this thread's output: long row fastest, then short row, item, chunk
+    const int ob = sh.items + sh.sb + sh.lr, outs = 1 << ob, o = tid & (outs - 1), g = tid >> ob;
+    const int l = o & (lr - 1), sr = (o >> sh.lr) & (S - 1), p = o >> (sh.lr + sh.sb);
+    float2 tot = make_float2(0.f, 0.f);
+    for (int k0 = 0; k0 < K; k0 += 1 << kt) {
+        if (k0) __syncthreads();
+        skinny_stage(ls, SWAP ? B : A, SWAP ? b_is : a_is, SWAP ? b_div : a_div, item0, np, SWAP ? bkm : akm, sh.lr,
+                     sh.kb, sh.lb, l0, k0, kt);
+        skinny_stage(ss, SWAP ? A : B, SWAP ? a_is : b_is, SWAP ? a_div : b_div, item0, np, SWAP ? akm : bkm, sh.sb,
+                     sh.kb, sh.sb, 0, k0, kt);
+        __syncthreads();
+        float2 acc = make_float2(0.f, 0.f);
+        if (g < G && p < np) {
+            const float2* lp = ls + (p * lr + l) * ld + (g << sh.kw);
+            const float2* sp = ss + (p * S + sr) * ld + (g << sh.kw);
+#pragma unroll 8
+            for (int k = 0; k < 1 << sh.kw; ++k) {
+                const float2 x = lp[k], y = sp[k];
+                cfma(acc, SWAP ? y : x, SWAP ? x : y);
+            }
+        }
+        if (G > 1) {
+            if (g < G) red[g * outs + o] = acc;
+            __syncthreads();
+            if (g == 0)
+                for (int c = 0; c < G; ++c) {
+                    const float2 v = red[c * outs + o];
+                    tot.x += v.x;
+                    tot.y += v.y;
+                }
+        } else {
+            tot.x += acc.x;
+            tot.y += acc.y;
+        }
+    }
+    if (g == 0 && p < np) {
+        const int64_t m = SWAP ? sr : l0 + l, n = SWAP ? l0 + l : sr;
+        const int nb = SWAP ? sh.lb : sh.sb;
+        float2* Cp = C + (item0 + p) * c_is;
+        Cp[om.on ? place_bits(m, om.pos + nb) + place_bits(n, om.pos) : (m << nb) + n] = tot;
+    }
+}
+
+static int skinny_smem(const SkinnyShape& sh) {
+    const int ld = (1 << (sh.g + sh.kw)) + 1;
+    return 8 * (((1 << sh.lr) + (1 << sh.sb)) * ld << sh.items) + (sh.g ? 8 << (sh.g + sh.items + sh.sb + sh.lr) : 0);
+}
+
+// the CTA shape of a skinny product, or false when it is not one
+static bool skinny_shape(int mb, int nb, int kb, SkinnyShape* sh) {
+    sh->lb = std::max(mb, nb);
+    sh->sb = std::min(mb, nb);
+    sh->kb = kb;
+    if (sh->sb > kSkinnyMax || kb < 3) return false;
+    sh->kw = std::min(kb, 6);
+    sh->lr = std::min(sh->lb, 8 - sh->sb);
+    sh->g = std::min(kb - sh->kw, 8 - sh->sb - sh->lr);
+    sh->items = 0;
+    while (skinny_smem(*sh) > kSkinnySmem && sh->g) --sh->g;
+    while (skinny_smem(*sh) > kSkinnySmem && sh->lr) --sh->lr;
+    if (sh->lr == sh->lb)  // whole items: as many as the threads left take
+        while (sh->items + sh->lr + sh->sb + sh->g < 8) {
+            ++sh->items;
+            if (skinny_smem(*sh) > kSkinnySmem) {
+                --sh->items;
+                break;
+            }
+        }
+    return skinny_smem(*sh) <= kSkinnySmem;
+}
+
+static cudaError_t gemm_skinny(const SkinnyShape& sh, bool swap, cudaStream_t st, const float2* a, int64_t a_is, bool akm,
+                               const float2* b, int64_t b_is, bool bkm, float2* c, int64_t c_is, int64_t n_items,
+                               const OutMap& om, int a_div, int b_div) {
+    const int smem = skinny_smem(sh);
+    {
+        static uint64_t done[2][4] = {};  // shared-memory opt-in, once per device and kernel
+        static std::mutex mu;
+        int dev = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e != cudaSuccess) return e;
+        std::lock_guard<std::mutex> lk(mu);
+        if (dev >= 256 || !((done[swap][dev >> 6] >> (dev & 63)) & 1)) {
+            e = cudaFuncSetAttribute(swap ? k_gemm_skinny<true> : k_gemm_skinny<false>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, kSkinnySmem);
+            if (e != cudaSuccess) return e;
+            if (dev < 256) done[swap][dev >> 6] |= 1ull << (dev & 63);
+        }
+    }
+    const dim3 grid(1u << (sh.lb - sh.lr), (unsigned)((n_items + (1 << sh.items) - 1) >> sh.items));
+    if (swap)
+        k_gemm_skinny<true><<<grid, 256, smem, st>>>(a, a_is, akm, b, b_is, bkm, c, c_is, sh, om, a_div, b_div, n_items);
+    else
+        k_gemm_skinny<false><<<grid, 256, smem, st>>>(a, a_is, akm, b, b_is, bkm, c, c_is, sh, om, a_div, b_div, n_items);
+    return cudaGetLastError();
+}
+
 // Long dot products (M * N <= 16 outputs, large K): one CTA per item, the 256
 // threads stride over K with a private partial per output, then a fixed-order
 // tree reduction (deterministic).
@@ -1128,6 +1287,10 @@ cudaError_t launch_gemm_c64(const float2* a, int64_t a_is, bool a_kmajor, const 
     const int bmb = mb >= 6 ? 6 : mb >= 5 ? 5 : 4;  // tile edge 64 / 32 / 16
     const int bnb = nb >= 6 ? 6 : nb >= 5 ? 5 : 4;
     const int64_t tm = ((1ll << mb) + (1 << bmb) - 1) >> bmb, tn = ((1ll << nb) + (1 << bnb) - 1) >> bnb;
+    SkinnyShape sh;  // see k_gemm_skinny for where the line lies
+    if ((std::min(mb, nb) <= 2 || mb + nb <= 6 || (kb >= 8 && tm * tn * n_items < 2 * sm_count())) &&
+        skinny_shape(mb, nb, kb, &sh))
+        return gemm_skinny(sh, mb < nb, st, a, a_is, a_kmajor, b, b_is, b_kmajor, c, c_is, n_items, om, a_div, b_div);
     dim3 grid((unsigned)(tm * tn), (unsigned)n_items);
 #define QX_GEMM_CASE(X, Y)                                                                            \
     if (bmb == X && bnb == Y) {                                                                       \
