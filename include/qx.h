@@ -100,7 +100,7 @@ typedef struct {
                                 the slice but on no output bit are computed
                                 once per slice and shared by the slice's
                                 bitstrings; 1: once per (slice, bitstring)
-                                pair, as executors 2 and 3 always do.  The
+                                pair, as the persistent kernel always does.  The
                                 amplitudes agree to FP32 rounding (launches
                                 over fewer items may pick other tiles). */
     int32_t pad;
@@ -377,10 +377,15 @@ int qx_esup_sample(qx_handle h, const uint8_t* d_candidates, const double* d_uni
  *   qx_group_bind    takes caller-owned device scratch of at least
  *                    qx_group_scratch_size bytes, uploads the members' tensors
  *                    and programs and synchronises the stream.
- *   qx_group_run     only enqueues: one launch for all members' invariant
- *                    tensors, one persistent launch for all (slice, bitstring)
- *                    pairs (largest programs first), one FP64 compensated sum
- *                    into the outputs.  No allocation, no host copies, no
+ *   qx_group_run     only enqueues: for the members with little work per
+ *                    pair one launch for all their invariant tensors, one
+ *                    persistent launch for all their (slice, bitstring) pairs
+ *                    (largest programs first) and one FP64 compensated sum
+ *                    into the outputs; the others (chosen at bind, where that
+ *                    is estimated faster) run one after another as launches
+ *                    over batches of pairs in the same scratch, per-slice
+ *                    steps once per slice.  The amplitudes are the same
+ *                    either way.  No allocation, no host copies, no
  *                    synchronisation, so a CUDA graph can capture it.
  * A group does not own its members; destroy it before them. */
 typedef struct qx_group* qx_group_t;

@@ -59,6 +59,7 @@ struct Storage {
     int level = 0;          // region: 0 invariant, 1 per slice, 2 per pair
     int64_t def = 0, last = 0;
     int64_t off = 0;        // entries within its region (per pair for the item region)
+    int64_t poff = 0;       // levels 1 and 2: entries within a persistent CTA's scratch
 };
 
 enum OpType { OP_PERM, OP_SMALL, OP_GEMM };
@@ -138,6 +139,7 @@ struct qx_ctx {
 
     // persistent executor program (variant ops, in order)
     bool persist_ok = false;
+    int64_t persist_entries = 0;  // scratch of one CTA: the tensors of a pair, per-slice ones among them
     std::vector<POp> pops;      // per-pair ops
     std::vector<POp> pops_inv;  // invariant ops (prologue program)
     PRef proot{};
@@ -167,6 +169,7 @@ struct qx_ctx {
     int n_waves = 0;
     bool segs_on = true;                // false: every step a launch of its own (workspaces too small for segments)
     std::vector<Storage> stor0;         // storages with the lifetimes of one launch per step
+    std::vector<std::pair<int64_t, int64_t>> pair_life;  // their lifetimes when a CTA runs one pair's steps in order
     bool wave_ok = false;               // there is a prologue launch
     std::vector<int> chain_of_op;       // per op: its prologue segment, -1 if none
     double wave_flops = 0, wave_bytes = 0;
@@ -438,11 +441,9 @@ static Node contiguous_node(const std::vector<int>& legs, int level, int storage
     return n;
 }
 
-// First-fit offsets for storages of one region (intervals [def, last] inclusive).
-static int64_t assign_offsets(qx_ctx* h, int level) {
-    std::vector<int> ids;
-    for (int i = 0; i < (int)h->stor.size(); ++i)
-        if (h->stor[i].level == level) ids.push_back(i);
+// First-fit offsets for the chosen storages (intervals [def, last] inclusive): ids in, the space they
+// take out.
+static int64_t first_fit(qx_ctx* h, std::vector<int> ids, int64_t Storage::*off) {
     std::sort(ids.begin(), ids.end(), [&](int a, int b) {
         if (h->stor[a].def != h->stor[b].def) return h->stor[a].def < h->stor[b].def;
         return a < b;
@@ -455,7 +456,7 @@ static int64_t assign_offsets(qx_ctx* h, int level) {
         std::vector<std::pair<int64_t, int64_t>> busy;
         for (int p : placed) {
             const Storage& o = h->stor[p];
-            if (o.last >= s.def && s.last >= o.def) busy.push_back({o.off, o.off + align_up(o.entries, kAlignEntries)});
+            if (o.last >= s.def && s.last >= o.def) busy.push_back({o.*off, o.*off + align_up(o.entries, kAlignEntries)});
         }
         std::sort(busy.begin(), busy.end());
         int64_t cand = 0;
@@ -463,9 +464,34 @@ static int64_t assign_offsets(qx_ctx* h, int level) {
             if (cand + need <= b.first) break;
             cand = std::max(cand, b.second);
         }
-        s.off = cand;
+        s.*off = cand;
         top = std::max(top, cand + need);
         placed.push_back(id);
+    }
+    return top;
+}
+// ... of one region
+static int64_t assign_offsets(qx_ctx* h, int level) {
+    std::vector<int> ids;
+    for (int i = 0; i < (int)h->stor.size(); ++i)
+        if (h->stor[i].level == level) ids.push_back(i);
+    return first_fit(h, ids, &Storage::off);
+}
+// ... of a persistent CTA's scratch: one pair's tensors, the per-slice ones among them (there a
+// per-slice tensor that pairs read need not outlive the pair: its own steps' lifetimes, stor0, do)
+static int64_t assign_scratch(qx_ctx* h) {
+    std::vector<int> ids;
+    std::vector<Storage> keep = h->stor;
+    for (int i = 0; i < (int)h->stor.size(); ++i)
+        if (h->stor[i].level > 0) {
+            ids.push_back(i);
+            h->stor[i].def = h->pair_life[i].first;
+            h->stor[i].last = h->pair_life[i].second;
+        }
+    const int64_t top = first_fit(h, ids, &Storage::poff);
+    for (int i : ids) {
+        h->stor[i].def = keep[i].def;
+        h->stor[i].last = keep[i].last;
     }
     return top;
 }
@@ -532,8 +558,8 @@ static int compile_plan(qx_ctx* h, const int64_t* order, int64_t n_steps, const 
                     (long long)n_steps, (long long)N, (long long)(N - 1));
     if (n_sliced < 0 || n_sliced > 40) return fail(h, QX_EINVAL, "n_sliced %d out of range [0, 40]", n_sliced);
     // Intermediates that depend on the slice but on no output bit are computed once per slice and
-    // shared by every bitstring of it (batched executor only).
-    const bool slice_level = h->opt.executor < 2 && !h->opt.no_slice_level;
+    // shared by every bitstring of it (the persistent kernel runs them once per pair).
+    const bool slice_level = h->opt.executor != 2 && !h->opt.no_slice_level;
     std::vector<int> fixsrc(h->n_bonds, INT32_MIN);  // source of each fixed bond
     for (int j = 0; j < n_sliced; ++j) {
         const int64_t e = sliced[j];
@@ -1088,6 +1114,8 @@ static int compile_plan(qx_ctx* h, const int64_t* order, int64_t n_steps, const 
         }
     }
     if (!R.variant && R.storage >= 0) h->stor[R.storage].last = kLive;
+    h->pair_life.clear();
+    for (const Storage& st : h->stor) h->pair_life.push_back({st.def, st.last});
     // per-slice storages read by per-pair work stay resident too, so that when a slice's bitstrings
     // need several batches of the per-pair region, the later batches run only the per-pair steps
     for (const Op& op : h->ops) {
@@ -1119,11 +1147,14 @@ static int compile_plan(qx_ctx* h, const int64_t* order, int64_t n_steps, const 
 // whose operands from outside live until the segment's last step (and whose results in the prologue
 // live from the start); without them every step is a launch of its own, which needs the least memory.
 static void finish_layout(qx_ctx* h, bool segs) {
-    h->segs_on = segs && h->opt.executor < 2;
+    h->segs_on = segs && h->opt.executor != 2;
     h->stor = h->stor0;
     choose_segments(h);
     h->item_entries = std::max<int64_t>(assign_offsets(h, 2), kAlignEntries);
     h->slice_entries = assign_offsets(h, 1);
+    if (h->opt.executor >= 2) {
+        h->persist_entries = std::max<int64_t>(assign_scratch(h), kAlignEntries);
+    }
     if (h->opt.executor < 2) {
         // a small invariant region gets no reuse: then the only hazards between invariant steps are
         // their data dependencies
@@ -1183,7 +1214,7 @@ static void layout(qx_ctx* h, int64_t max_bits, int64_t* fixed_bytes) {
     if (persist_active(h)) {
         off += 256;
         h->off_pscratch = off;
-        off += align_up((int64_t)h->persist_grid * h->item_entries * 8, 256);
+        off += align_up((int64_t)h->persist_grid * h->persist_entries * 8, 256);
     }
     h->off_wave = off;  // segment programs
     off += align_up((int64_t)h->seg_blob.size(), 256);
@@ -1219,13 +1250,30 @@ static bool fit_regions(const qx_ctx* h, int64_t avail, int64_t max_bits, int64_
 static bool fit_layout(qx_ctx* h, int64_t bytes, const int64_t* batch_bytes, int64_t max_bits, int64_t* fixed,
                        int64_t* items, int64_t* slices) {
     for (bool segs : {true, false}) {
-        if (h->opt.executor < 2 && h->segs_on != segs) finish_layout(h, segs);
+        if (h->opt.executor != 2 && h->segs_on != segs) finish_layout(h, segs);
         layout(h, max_bits, fixed);
+        if (h->opt.executor == 3) {  // a group member's own batch region is one pair's, its group's scratch serves runs
+            *items = *slices = 1;
+            if (bytes - *fixed >= h->persist_entries * 8) return true;
+            continue;
+        }
         const bool room = !batch_bytes || *fixed <= bytes;
         if (room && fit_regions(h, batch_bytes ? *batch_bytes : bytes - *fixed, max_bits, items, slices)) return true;
-        if (h->opt.executor >= 2) return false;
+        if (h->opt.executor == 2) return false;
     }
     return false;
+}
+
+// The same for calls of exactly n_bits bitstrings: whole slices, each with all its bitstrings and one
+// copy of the per-slice tensors, as long as one such slice fits.
+static bool fit_whole_slices(const qx_ctx* h, int64_t avail, int64_t n_bits, int64_t* items_out, int64_t* slices_out) {
+    int64_t ns = (avail - 512) / ((h->slice_entries + n_bits * h->item_entries) * 8);
+    ns = std::min(ns, std::min(h->n_slices, kMaxBatchItems / n_bits));
+    if (h->opt.max_items > 0) ns = std::min(ns, h->opt.max_items / n_bits);
+    if (ns < 1) return fit_regions(h, avail, n_bits, items_out, slices_out);
+    *items_out = ns * n_bits;
+    *slices_out = h->slice_entries ? ns : 0;
+    return true;
 }
 
 // Region offsets for a workspace whose fixed part ends at `fixed`.
@@ -1364,7 +1412,7 @@ static PRef pref_node(const qx_ctx* h, int node) {
     } else {
         const Storage& st = h->stor[nd.storage];
         r.space = st.variant ? PSPACE_SCRATCH : PSPACE_INV;
-        r.off = st.off;
+        r.off = st.variant ? st.poff : st.off;
     }
     return r;
 }
@@ -1373,7 +1421,7 @@ static PRef pref_storage(const qx_ctx* h, int sid) {
     const Storage& st = h->stor[sid];
     PRef r{};
     r.space = st.variant ? PSPACE_SCRATCH : PSPACE_INV;
-    r.off = st.off;
+    r.off = st.variant ? st.poff : st.off;
     return r;
 }
 
@@ -1382,7 +1430,7 @@ static POp to_pop(const qx_ctx* h, const Op& op) {
     p.mb = op.mb;
     p.kb = op.kb;
     p.nb = op.nb;
-    p.dst = h->stor[op.dst].off;
+    p.dst = op.variant ? h->stor[op.dst].poff : h->stor[op.dst].off;
     if (op.type == OP_PERM) {
         const PermDesc d = perm_desc(h, op, 5, 10);  // the persistent kernel's tiles: 2^10 entries, 5 + 5 bits
         p.type = POP_PERM;
@@ -1415,10 +1463,11 @@ static POp to_pop(const qx_ctx* h, const Op& op) {
 
 static void build_persistent_program(qx_ctx* h) {
     h->persist_ok = false;
+    if (h->opt.executor < 2) return;
     h->pops.clear();
     h->pops_inv.clear();
     for (const Op& op : h->ops)
-        if (op.tc || !op.out_pos.empty() || op.dot_perm || op.level == 1) return;  // these run batched only
+        if (op.tc || !op.out_pos.empty() || op.dot_perm) return;  // these run batched only
     const Node& R = h->nodes[h->root];
     if (!R.variant) return;  // nothing depends on the pair
     // invariant ops write the invariant region: their program runs with that region as scratch
@@ -1982,6 +2031,15 @@ static int upload_programs(qx_ctx* h) {
     return QX_OK;
 }
 
+static int upload_segments(qx_ctx* h) {
+    if (h->segs_on_device || h->seg_blob.empty()) return QX_OK;
+    CUDA_TRY(h, cudaMemcpyAsync(h->ws + h->off_wave, h->seg_blob.data(), h->seg_blob.size(), cudaMemcpyHostToDevice,
+                                h->stream));
+    CUDA_TRY(h, cudaStreamSynchronize(h->stream));
+    h->segs_on_device = true;
+    return QX_OK;
+}
+
 // the pair program (inv = true: the prologue program) of a handle, for slices [s_begin, s_end)
 static PProg make_prog(const qx_ctx* h, bool inv, const uint8_t* d_bits, int64_t n_bits, int64_t s_begin) {
     PProg g{};
@@ -2023,7 +2081,7 @@ static int contract_persistent(qx_ctx* h, const uint8_t* d_bits, int64_t n_bits,
     PLaunch L{};
     L.n_progs = 0;
     L.scratch = (float2*)(h->ws + h->off_pscratch);
-    L.scratch_entries = h->item_entries;
+    L.scratch_entries = h->persist_entries;
     L.counter = (unsigned long long*)(h->ws + h->off_counter);
     size_t slot;
     cudaError_t e = cudaSuccess;
@@ -2042,12 +2100,12 @@ static int contract_persistent(qx_ctx* h, const uint8_t* d_bits, int64_t n_bits,
     double bytes = 0;
     for (const Op& op : h->ops)
         if (op.variant) bytes += op_bytes(h, op, pairs);
-    e = prof_begin(h, QX_KERNEL_PERSIST, h->flops_item * (double)pairs, bytes, &slot);
+    e = prof_begin(h, QX_KERNEL_PERSIST, (h->flops_slice + h->flops_item) * (double)pairs, bytes, &slot);
     if (e == cudaSuccess) e = launch_persist(L, h->persist_grid, h->stream);
     if (e == cudaSuccess) e = prof_end(h, slot);
     if (e != cudaSuccess) return fail(h, QX_ECUDA, "persistent launch failed: %s", cudaGetErrorString(e));
     h->last_launches += 1;
-    h->last_flops += h->flops_item * (double)pairs;
+    h->last_flops += (h->flops_slice + h->flops_item) * (double)pairs;
     // deterministic FP64 sum over the slices of each bitstring, straight into the amplitudes
     const int64_t n_o = (int64_t)1 << n_open(h);
     const GSum g = make_gsum(h, n_bits, s_end - s_begin, d_amps, 0);
@@ -2232,8 +2290,9 @@ struct Dag {
     }
 };
 
+// in_group: a member of a group whose steps run as launches over batches (qx_group_run)
 static int contract_impl(qx_ctx* h, const uint8_t* d_bits, int64_t n_bits, int64_t s_begin, int64_t s_end,
-                         double* d_amps) {
+                         double* d_amps, bool in_group = false) {
     const int64_t n_o = (int64_t)1 << n_open(h);
     h->last_flops = 0;
     h->last_launches = 0;
@@ -2245,15 +2304,10 @@ static int contract_impl(qx_ctx* h, const uint8_t* d_bits, int64_t n_bits, int64
         CUDA_TRY(h, cudaStreamSynchronize(h->stream));
         h->leaves_on_device = true;
     }
-    if (!h->segs_on_device && !h->seg_blob.empty()) {
-        CUDA_TRY(h, cudaMemcpyAsync(h->ws + h->off_wave, h->seg_blob.data(), h->seg_blob.size(),
-                                    cudaMemcpyHostToDevice, h->stream));
-        CUDA_TRY(h, cudaStreamSynchronize(h->stream));
-        h->segs_on_device = true;
-    }
+    if (const int rc = upload_segments(h)) return rc;
     double* acc = (double*)(h->ws + h->off_acc);
     CUDA_TRY(h, cudaMemsetAsync(h->ws + h->off_err, 0, sizeof(int), h->stream));
-    const int mode = h->opt.executor;
+    const int mode = in_group ? 1 : h->opt.executor;
     if (mode >= 2 && !persist_active(h))
         return fail(h, QX_EINVAL, mode == 3 ? "a group member contracts only through qx_group_run"
                                             : "the persistent executor does not apply to this plan and precision form");
@@ -2516,6 +2570,10 @@ int qx_workspace_size(qx_handle h, int64_t max_bits, int64_t items, int64_t* byt
     if (items < 1) items = 1;
     int64_t fixed;
     layout(h, max_bits, &fixed);
+    if (h->opt.executor == 3) {
+        *bytes_out = fixed + items * h->persist_entries * 8;
+        return QX_OK;
+    }
     const int64_t slices = h->slice_entries ? std::min<int64_t>(h->n_slices, items) : 0;
     *bytes_out = fixed + align_up(slices * h->slice_entries * 8, 256) + items * h->item_entries * 8;
     return QX_OK;
@@ -2531,7 +2589,7 @@ int qx_bind_workspace(qx_handle h, void* dptr, int64_t bytes, int64_t max_bits) 
     int64_t fixed, items = 0, slices = 0;
     if (!fit_layout(h, bytes, nullptr, max_bits, &fixed, &items, &slices))
         return fail(h, QX_ENOMEM, "workspace of %lld bytes holds no (slice, bitstring) pair; need %lld", (long long)bytes,
-                    (long long)(fixed + 256 + (h->item_entries + h->slice_entries) * 8));
+                    (long long)(fixed + 256 + (h->opt.executor == 3 ? h->persist_entries : h->item_entries + h->slice_entries) * 8));
     CUDA_TRY(h, cudaSetDevice(h->device));
     if (!dptr) {
         CUDA_TRY(h, cudaMalloc(&dptr, (size_t)bytes));
@@ -3031,12 +3089,111 @@ struct qx_group {
     int64_t off_inv = 0, off_pair = 0, off_sum = 0, off_sc = 0;
     std::string err;
     bool bound = false;
+    // members whose steps run as launches over batches of pairs instead of in the persistent launch:
+    // their batch regions lie in the persistent launch's scratch, and they share these streams and events
+    struct Batched { int member; int64_t items, slices; };
+    std::vector<Batched> batched;
+    std::vector<cudaStream_t> dstreams;
+    std::vector<cudaEvent_t> op_ev, join_ev;
+    cudaEvent_t fork_ev = nullptr, wave_ev = nullptr;
 };
+
+// Estimated microseconds of a member on the persistent launch (its share of the GPU) and as launches.
+// The persistent kernel runs one pair per CTA, per-slice steps included, at about 12 TFLOP/s over the
+// GPU; launches cost 2.5 us each per batch, their flops at 35 TFLOP/s or their bytes at 4.5 TB/s.
+static double persist_us(const qx_ctx* h, int64_t n_bits) {
+    return (double)(h->n_slices * n_bits) * (h->flops_slice + h->flops_item) / 12e6;
+}
+static double batched_us(const qx_ctx* h, int64_t n_bits, int64_t items, int64_t slices) {
+    const int64_t nb = std::min(items, n_bits);
+    int64_t ns = items >= n_bits ? std::min(h->n_slices, items / n_bits) : 1;
+    if (h->slice_entries) ns = std::max<int64_t>(1, std::min(ns, slices));
+    const int64_t at_once[3] = {1, ns, ns * nb};
+    const double bit_batches = (double)((n_bits + nb - 1) / nb), slice_batches = (double)((h->n_slices + ns - 1) / ns);
+    const double times[3] = {1.0, slice_batches, slice_batches * bit_batches};
+    std::vector<char> in_seg(h->ops.size(), 0);
+    double us = h->wave_ok ? 15.0 : 0.0;
+    for (const auto& sg : h->segs) {
+        if (!sg.wave && !seg_pays(sg, at_once[sg.level])) continue;
+        for (int j : sg.ops) in_seg[j] = 1;
+        if (!sg.wave) us += times[sg.level] * (4.0 + 0.35 * sg.n_stages);
+    }
+    for (size_t j = 0; j < h->ops.size(); ++j) {
+        if (in_seg[j]) continue;
+        const Op& op = h->ops[j];
+        const double n = (double)at_once[op.level];
+        us += times[op.level] * std::max(2.5, std::max(op.flops * n / 35e6, op_bytes(h, op, (int64_t)n, nb) / 4.5e6));
+    }
+    return us + 10.0 * times[2];
+}
 
 static int gfail(qx_group* g, int code, const char* msg) {
     g->err = msg;
     return code;
 }
+
+// the streams and events of the batched members (made at bind: a run may be captured)
+static cudaError_t group_streams(qx_group* g, size_t n_ops) {
+    cudaError_t e = cudaSuccess;
+    auto event = [&](cudaEvent_t* ev) { return cudaEventCreateWithFlags(ev, cudaEventDisableTiming); };
+    while (e == cudaSuccess && g->dstreams.size() < 7) {
+        cudaStream_t st;
+        if ((e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking)) == cudaSuccess) g->dstreams.push_back(st);
+    }
+    for (auto* v : {&g->join_ev, &g->op_ev})
+        while (e == cudaSuccess && v->size() < (v == &g->join_ev ? 7 : n_ops)) {
+            cudaEvent_t ev;
+            if ((e = event(&ev)) == cudaSuccess) v->push_back(ev);
+        }
+    if (e == cudaSuccess && !g->fork_ev) e = event(&g->fork_ev);
+    if (e == cudaSuccess && !g->wave_ev) e = event(&g->wave_ev);
+    return e;
+}
+
+// A batched member for the time of one run: its handle on the group's stream, streams, events and
+// scratch, without the state of other calls (kept invariants, profiling); all put back afterwards.
+struct BatchedMember {
+    qx_group* g;
+    qx_ctx* h;
+    cudaStream_t stream;
+    char* wb;
+    int64_t off_slice, off_item, items_cap, slices_cap;
+    bool memo, profiling, clear, final_;
+    int n_streams;
+    void trade() {
+        std::swap(h->dstreams, g->dstreams);
+        std::swap(h->join_ev, g->join_ev);
+        std::swap(h->op_ev, g->op_ev);
+        std::swap(h->fork_ev, g->fork_ev);
+        std::swap(h->wave_ev, g->wave_ev);
+    }
+    BatchedMember(qx_group* gg, qx_ctx* hh, const qx_group::Batched& b)
+        : g(gg), h(hh), stream(hh->stream), wb(hh->wb), off_slice(hh->off_slice), off_item(hh->off_item),
+          items_cap(hh->items_cap), slices_cap(hh->slices_cap), memo(hh->memo), profiling(hh->profiling),
+          clear(hh->part_clear), final_(hh->part_final), n_streams(hh->n_streams) {
+        trade();
+        h->stream = g->stream;
+        h->wb = g->scratch + g->off_sc;
+        place_regions(h, 0, b.items, b.slices);
+        h->memo = h->profiling = false;
+        h->part_clear = h->part_final = true;
+        h->n_streams = std::min(n_streams, 8);
+    }
+    ~BatchedMember() {
+        trade();
+        h->stream = stream;
+        h->wb = wb;
+        h->off_slice = off_slice;
+        h->off_item = off_item;
+        h->items_cap = items_cap;
+        h->slices_cap = slices_cap;
+        h->memo = memo;
+        h->profiling = profiling;
+        h->part_clear = clear;
+        h->part_final = final_;
+        h->n_streams = n_streams;
+    }
+};
 
 static void group_layout(qx_group* g, int64_t* bytes) {
     int64_t off = 256;  // work counter
@@ -3079,7 +3236,7 @@ int qx_group_create(qx_group_t* out, qx_handle* hs, int32_t n, const uint8_t* co
         g->bits.push_back(d_bits[i]);
         g->n_bits.push_back(n_bits[i]);
         g->amps.push_back(d_amps[i]);
-        g->max_entries = std::max(g->max_entries, h->item_entries);
+        g->max_entries = std::max(g->max_entries, h->persist_entries);
     }
     g->device = hs[0]->device;
     g->stream = hs[0]->stream;
@@ -3114,19 +3271,39 @@ int qx_group_bind(qx_group_t g, void* d_scratch, int64_t bytes) {
                 return gfail(g, QX_ECUDA, "leaf upload failed");
             h->leaves_on_device = true;
         }
-        if (upload_programs(h) != QX_OK) return gfail(g, QX_ECUDA, h->err.c_str());
+        if (upload_programs(h) != QX_OK || upload_segments(h) != QX_OK) return gfail(g, QX_ECUDA, h->err.c_str());
     }
+    // which members run as launches: those estimated faster so, where a batch fits the scratch
+    g->batched.clear();
+    std::vector<char> as_launches(g->hs.size(), 0);
+    const int64_t room = (int64_t)g->grid * g->max_entries * 8;
+    size_t max_ops = 0;
+    for (size_t i = 0; i < g->hs.size(); ++i) {
+        qx_ctx* h = g->hs[i];
+        int64_t items = 0, slices = 0;
+        if (!fit_whole_slices(h, room, g->n_bits[i], &items, &slices) ||
+            batched_us(h, g->n_bits[i], items, slices) >= persist_us(h, g->n_bits[i]))
+            continue;
+        as_launches[i] = 1;
+        g->batched.push_back({(int)i, items, slices});
+        max_ops = std::max(max_ops, h->ops.size());
+    }
+    if (!g->batched.empty() && group_streams(g, max_ops) != cudaSuccess)
+        return gfail(g, QX_ECUDA, "stream or event creation failed");
     // programs ordered by per-pair work, largest first, so the long pairs start early
     std::vector<int> order(g->hs.size());
     for (size_t i = 0; i < order.size(); ++i) order[i] = (int)i;
     std::stable_sort(order.begin(), order.end(),
-                     [&](int a, int b) { return g->hs[a]->flops_item > g->hs[b]->flops_item; });
+                     [&](int a, int b) {
+                         return g->hs[a]->flops_slice + g->hs[a]->flops_item > g->hs[b]->flops_slice + g->hs[b]->flops_item;
+                     });
     g->inv_progs.clear();
     g->pair_progs.clear();
     g->sums.clear();
     int64_t w = 0, t = 0;
     for (int i : order) {
         qx_ctx* h = g->hs[i];
+        if (as_launches[i]) continue;
         if (!h->pops_inv.empty()) {
             PProg p = make_prog(h, true, g->bits[i], 1, 0);
             p.work0 = (int64_t)g->inv_progs.size();
@@ -3139,6 +3316,7 @@ int qx_group_bind(qx_group_t g, void* d_scratch, int64_t bytes) {
     }
     for (size_t i = 0; i < g->hs.size(); ++i) {
         qx_ctx* h = g->hs[i];
+        if (as_launches[i]) continue;
         g->sums.push_back(make_gsum(h, g->n_bits[i], h->n_slices, g->amps[i], t));
         t += g->n_bits[i] << n_open(h);
     }
@@ -3148,10 +3326,10 @@ int qx_group_bind(qx_group_t g, void* d_scratch, int64_t bytes) {
     if (!g->inv_progs.empty())
         e = cudaMemcpyAsync(g->scratch + g->off_inv, g->inv_progs.data(), g->inv_progs.size() * sizeof(PProg),
                             cudaMemcpyHostToDevice, g->stream);
-    if (e == cudaSuccess)
+    if (e == cudaSuccess && !g->pair_progs.empty())
         e = cudaMemcpyAsync(g->scratch + g->off_pair, g->pair_progs.data(), g->pair_progs.size() * sizeof(PProg),
                             cudaMemcpyHostToDevice, g->stream);
-    if (e == cudaSuccess)
+    if (e == cudaSuccess && !g->sums.empty())
         e = cudaMemcpyAsync(g->scratch + g->off_sum, g->sums.data(), g->sums.size() * sizeof(GSum),
                             cudaMemcpyHostToDevice, g->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(g->stream);
@@ -3175,7 +3353,7 @@ int qx_group_run(qx_group_t g) {
         L.n_work = L.n_progs;
         e = launch_persist(L, std::min<int>(g->grid, L.n_progs), g->stream);
     }
-    if (e == cudaSuccess) {
+    if (e == cudaSuccess && !g->pair_progs.empty()) {
         L.progs = (const PProg*)(g->scratch + g->off_pair);
         L.n_progs = (int32_t)g->pair_progs.size();
         L.n_work = g->n_pair_work;
@@ -3184,9 +3362,23 @@ int qx_group_run(qx_group_t g) {
     if (e == cudaSuccess)
         e = launch_group_sum((const GSum*)(g->scratch + g->off_sum), (int32_t)g->sums.size(), g->total_sum, g->stream);
     if (e != cudaSuccess) return gfail(g, QX_ECUDA, cudaGetErrorString(e));
+    for (const auto& b : g->batched) {
+        qx_ctx* h = g->hs[b.member];
+        BatchedMember in(g, h, b);
+        if (contract_impl(h, g->bits[b.member], g->n_bits[b.member], 0, h->n_slices, g->amps[b.member], true) != QX_OK)
+            return gfail(g, QX_ECUDA, h->err.c_str());
+    }
     return QX_OK;
 }
 
-void qx_group_destroy(qx_group_t g) { delete g; }
+void qx_group_destroy(qx_group_t g) {
+    if (!g) return;
+    for (cudaEvent_t e : g->op_ev) cudaEventDestroy(e);
+    for (cudaEvent_t e : g->join_ev) cudaEventDestroy(e);
+    if (g->fork_ev) cudaEventDestroy(g->fork_ev);
+    if (g->wave_ev) cudaEventDestroy(g->wave_ev);
+    for (cudaStream_t st : g->dstreams) cudaStreamDestroy(st);
+    delete g;
+}
 
 }  // extern "C"
