@@ -61,7 +61,7 @@ struct TcForm<TC_FORM_BF16X3> {
 template <>
 struct TcForm<TC_FORM_FP16> {
     using T = __half;
-    static constexpr int NPA = 1, NPB = 1, NPROD = 1, EB = 2, FMT = 0, STAGES = 6;
+    static constexpr int NPA = 1, NPB = 1, NPROD = 1, EB = 2, FMT = 0, STAGES = 5;  // + the store blocks: 192 KB
     static __device__ __forceinline__ int pa(int) { return 0; }
     static __device__ __forceinline__ int pb(int) { return 0; }
 };
@@ -234,27 +234,54 @@ __device__ __forceinline__ void tc_commit(uint64_t* b) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(s_addr(b))
                  : "memory");
 }
-// Partial in-register transpose of a 32 x 32 block held one row per lane (a[i] = element (lane, i)):
-// register index bits 2..4 trade places with lane bits 0..2, one exchange with lane ^ 2^t per
-// register pair for t = 0, 1, 2.  Afterwards a[4 r + c] of lane l is element (8 (l >> 3) + r,
-// 4 (l & 7) + c): each register quad is four consecutive columns of one row, so one 16-byte store
-// per quad from the 32 lanes writes four whole 128-byte row runs (three exchange rounds and eight
-// stores instead of five rounds and 32 stores of a full transpose).
-__device__ __forceinline__ void transpose_q4(float* a, int lane) {
+// Writes 32 NB columns of 32 rows, one row per lane in v, to C at column x, row y, item z: 32 columns at a
+// time through the warp's 4 KB blocks of shared memory (128-byte rows, swizzled as the tensor map says, so
+// the lanes' 16-byte stores do not conflict) and out by one TMA store of whole 128-byte lines.  The
+// drain warps' instruction stream bounds the short-K products, and exchanging values across the lanes
+// for coalesced stores took about 300 of an epilogue's 500 instructions; 32-byte stores straight from
+// the lanes write 32 lines an instruction, which the memory-bound products do not like (4.8 TB/s).
+// Exchange -> here, one landing slot fewer for the blocks (us): 2^14 x 64 x 64, B shared, 376 items
+// 1193 -> 1026 (6.15 TB/s); B per item 1474 -> 1233; 2048 x 256 x 32 499 -> 361; 4096 x 64 x 32 257 -> 196; 2048 x
+// 512 x 512 on pre-split operands 3065 -> 2890 (188 items).  Only 2^15 x 32 x 32 with A read K-major is
+// slower (906 -> 972; gathered, as plans read it, 1278 -> 1202).
+constexpr int kEpiBytes = 4096;
+template <int NB, int NBUF = 1>
+__device__ __forceinline__ void store_rows(uint8_t* blocks, const CUtensorMap* map, const float* v, int x, int y, int z,
+                                           int lane) {
 #pragma unroll
-    for (int t = 0; t < 3; ++t) {
-        const int p = 2 + t;
-        const bool up = (lane >> t) & 1;
+    for (int b = 0; b < NB; ++b) {
+        // the block that used this buffer before is out (NBUF blocks of 4 KB are used in turn)
+        if (lane == 0) asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(NBUF - 1) : "memory");
+        __syncwarp();
+        uint8_t* stage = blocks + (b % NBUF) * kEpiBytes;
 #pragma unroll
-        for (int i = 0; i < 32; ++i) {
-            if ((i >> p) & 1) continue;
-            const int j = i | (1 << p);
-            const float send = up ? a[i] : a[j];
-            const float recv = __shfl_xor_sync(0xffffffffu, send, 1 << t);
-            if (up) a[i] = recv;
-            else a[j] = recv;
+        for (int j = 0; j < 8; ++j)
+            *(float4*)(stage + lane * 128 + ((j ^ (lane & 7)) << 4)) =
+                make_float4(v[32 * b + 4 * j], v[32 * b + 4 * j + 1], v[32 * b + 4 * j + 2], v[32 * b + 4 * j + 3]);
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) {
+            asm volatile(
+                "cp.async.bulk.tensor.3d.global.shared::cta.tile.bulk_group [%0, {%1, %2, %3}], [%4];" ::"l"((uint64_t)map),
+                "r"(x + 32 * b), "r"(y), "r"(z), "r"(s_addr(stage))
+                : "memory");
+            asm volatile("cp.async.bulk.commit_group;" ::: "memory");
         }
     }
+}
+// before a warp that used store_rows exits: its stores are done
+__device__ __forceinline__ void store_rows_end(int lane) {
+    if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+}
+// t[i] += v[i], two at a time (the same roundings)
+template <int N>
+__device__ __forceinline__ void add_row(float* t, const float* v) {
+#pragma unroll
+    for (int j = 0; j < N; j += 2)
+        asm("{\n\t.reg .b64 a, b;\n\tmov.b64 a, {%0, %1};\n\tmov.b64 b, {%2, %3};\n\tadd.rn.f32x2 a, a, b;\n\t"
+            "mov.b64 {%0, %1}, a;\n\t}\n"
+            : "+f"(t[j]), "+f"(t[j + 1])
+            : "f"(v[j]), "f"(v[j + 1]));
 }
 
 // 128-byte-swizzled K-major operand tile: rows of 128 B, 8-row groups 1024 B apart
@@ -345,6 +372,7 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
 struct TcMaps {
     CUtensorMap a[3];
     CUtensorMap b[3];
+    CUtensorMap c;
 };
 
 // ------------------------------------------------------------------------------------------------
@@ -362,6 +390,8 @@ struct TcTile {
     static constexpr int EW = BN / 32;                             // epilogue warps
     static constexpr int THREADS = 64 + 32 * EW;
     static constexpr int NTB = 512 / BN;                          // TMEM accumulator buffers
+    // store blocks per epilogue warp: two where the ring leaves the room (small kernels share the SM's rest)
+    static constexpr int EBUF = FORM == TC_FORM_FP16 && BN == 128 ? 2 : 1;
     static constexpr uint32_t TILE_A = TC_BM * ROWB, TILE_B = BN * ROWB;
     static constexpr uint32_t STAGE_BYTES = F::NPA * TILE_A + F::NPB * TILE_B;
     static constexpr int STAGES = BN == 128 && ROWB == 128 ? F::STAGES : (int)(TC_SMEM_LIMIT / STAGE_BYTES);
@@ -369,7 +399,7 @@ struct TcTile {
 
 template <int FORM, int BN, int ROWB>
 __global__ void __launch_bounds__(TcTile<FORM, BN, ROWB>::THREADS, 1)
-    k_gemm_tc(const __grid_constant__ TcMaps maps, float* __restrict__ C, int64_t c_is, int M, int N2, int K2,
+    k_gemm_tc(const __grid_constant__ TcMaps maps, int K2,
               int tiles_n, int tiles, int64_t n_items, long long limit, int* err, const float* amax, int a_div,
               int b_div) {
     // persistent over (item, tile) jobs: job = blockIdx.x + t * gridDim.x, tiles of an item in order (n
@@ -537,8 +567,7 @@ __global__ void __launch_bounds__(TcTile<FORM, BN, ROWB>::THREADS, 1)
                 for (int c = 0; c < 4; ++c) {
                     float v[32];
                     tmem_ld32(tmem + ((uint32_t)(32 * q) << 16) + b * BN + 128 * h + 32 * c, v);
-#pragma unroll
-                    for (int jj = 0; jj < 32; ++jj) tot[32 * c + jj] += v[jj];
+                    add_row<32>(tot + 32 * c, v);
                 }
                 tc_fence_before();
                 __syncwarp();
@@ -554,18 +583,10 @@ __global__ void __launch_bounds__(TcTile<FORM, BN, ROWB>::THREADS, 1)
             // tiles are whole (rows and columns multiples of 128; see tc_shape_ok)
             int item, m0, n0;
             job_of(t, &item, &m0, &n0);
-            float* cb = C + (int64_t)item * c_is + (int64_t)(m0 + 32 * q + ((lane >> 3) << 3)) * N2 + n0 + 128 * h +
-                        ((lane & 7) << 2);
-#pragma unroll
-            for (int b32 = 0; b32 < 4; ++b32) {
-                float* tt = tot + 32 * b32;
-                transpose_q4(tt, lane);
-#pragma unroll
-                for (int r = 0; r < 8; ++r)
-                    *(float4*)(cb + (int64_t)r * N2 + 32 * b32) =
-                        make_float4(tt[4 * r], tt[4 * r + 1], tt[4 * r + 2], tt[4 * r + 3]);
-            }
+            store_rows<4, T::EBUF>(base + STAGES * STAGE_BYTES + (warp - 2) * T::EBUF * kEpiBytes, &maps.c, tot, n0 + 128 * h, m0 + 32 * q,
+                          item, lane);
         }
+        store_rows_end(lane);
     }
     tc_fence_before();
     __syncthreads();
@@ -605,8 +626,9 @@ struct Tc2 {
     static constexpr uint32_t A = 16384, BRAW = (BN / 2) * 128, BP = BN * 128;
     static constexpr uint32_t LAND = A + BRAW;          // landing slot: raw A, raw B
     static constexpr uint32_t OFF_BLO = BP, MSLOT = 2 * BP;  // MMA slot: B' hi, B' lo
-    static constexpr int NL = BN == 128 ? 5 : 8, NM = BN == 128 ? 3 : 4;
-    static constexpr uint32_t SMEM = NL * LAND + NM * MSLOT;  // slots are multiples of 1024 bytes
+    static constexpr int NL = BN == 128 ? 4 : 6, NM = BN == 128 ? 3 : 4;
+    static constexpr uint32_t RINGS = NL * LAND + NM * MSLOT;  // slots are multiples of 1024 bytes
+    static constexpr uint32_t SMEM = RINGS + 8 * kEpiBytes;    // and the drain warps' store blocks
     static constexpr int NTB = 2;                      // accumulator buffers
     static constexpr uint32_t ACOL = NTB * BN;         // first TMEM column of the A parts (64 per MMA slot)
     static constexpr uint32_t TMEM_COLS = 512;
@@ -676,7 +698,7 @@ __device__ __forceinline__ void tc2_convert(const uint8_t* land, uint8_t* ms, in
 template <int BN>
 __global__ void __launch_bounds__(TC2_THREADS2, 1)
     k_gemm_tc2(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
-               float* __restrict__ C, int64_t c_is, int M, int N2, int K2, int tiles_n, int tiles, int64_t n_items,
+               const __grid_constant__ CUtensorMap mapC, int K2, int tiles_n, int tiles, int64_t n_items,
                int a_div, int b_div, int keep_a, int pack2, long long limit, int* err) {
     // persistent over (pair, tile) jobs: job = blockIdx.x + t * gridDim.x; the
     // k-stages of successive jobs form one sequence g = t * nk + it, so both
@@ -929,8 +951,7 @@ __global__ void __launch_bounds__(TC2_THREADS2, 1)
                 for (int c = 0; c < BN / 32; ++c) {  // 16 columns at a time (registers: 608 threads)
                     float v[16];
                     tmem_ld16(tmem + ((uint32_t)(32 * q) << 16) + b * BN + (BN / 2) * half + 16 * c, v);
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) tot[16 * c + j] += v[j];
+                    add_row<16>(tot + 16 * c, v);
                 }
                 tc_fence_before();
                 __syncwarp();
@@ -942,22 +963,13 @@ __global__ void __launch_bounds__(TC2_THREADS2, 1)
             int64_t item, akey;
             int m0, n0;
             job_of(t, &item, &m0, &n0, &akey);
-            // lane r holds row 32 q + r; each 32-column block is partly transposed across the warp so
-            // that every 16-byte store instruction writes whole 128-byte runs of four rows
-            float* cb = (pack2 ? C + (item + half) * c_is : C + item * c_is + n0 + (BN / 2) * half) +
-                        (int64_t)(m0 + 32 * q + ((lane >> 3) << 3)) * N2 + ((lane & 7) << 2);
+            // lane r holds row 32 q + r
+            store_rows<BN / 64>(base + L::RINGS + (warp - 2) * kEpiBytes, &mapC, tot, pack2 ? 0 : n0 + (BN / 2) * half,
+                                m0 + 32 * q, (int)(pack2 ? item + half : item), lane);
 #pragma unroll
-            for (int b32 = 0; b32 < BN / 64; ++b32) {
-                float* t = tot + 32 * b32;
-                transpose_q4(t, lane);
-#pragma unroll
-                for (int r = 0; r < 8; ++r) {
-                    *(float4*)(cb + (int64_t)r * N2 + 32 * b32) =
-                        make_float4(t[4 * r], t[4 * r + 1], t[4 * r + 2], t[4 * r + 3]);
-                    t[4 * r] = t[4 * r + 1] = t[4 * r + 2] = t[4 * r + 3] = 0.f;
-                }
-            }
+            for (int j = 0; j < BN / 2; ++j) tot[j] = 0.f;
         }
+        store_rows_end(lane);
     }
     tc_fence_before();
     __syncthreads();
@@ -975,8 +987,7 @@ __global__ void __launch_bounds__(TC2_THREADS2, 1)
 // (2N = BN), with at most Tc2Kb::MAXK k-stages: B' (hi and lo) of every stage is built once per CTA
 // and stays in shared memory, so per job TMA brings only A and the converter warps only split A into
 // TMEM -- half the converter work and no B traffic per job.  Roles and rings otherwise as in
-// k_gemm_tc2 with one converter group: warps 0 TMA, 1 and 14 MMA (even / odd stages), 2-9 drain,
-// 10-13 convert.
+// k_gemm_tc2: warps 0 TMA, 1 and 14 MMA (even / odd stages), 2-9 drain, 10-13 and 15-18 convert.
 // ------------------------------------------------------------------------------------------------
 template <int BN>
 struct Tc2Kb {
@@ -984,8 +995,9 @@ struct Tc2Kb {
     static constexpr uint32_t LAND = A;                      // landing slot: a raw A slab (first: raw B)
     static constexpr uint32_t OFF_BLO = BP, BSLOT = 2 * BP;  // resident B' of one stage: hi, lo
     static constexpr int MAXK = BN == 128 ? 4 : 8;           // k-stages whose B' stays resident
-    static constexpr int NL = 5, NM = 3;                     // landing slots; A positions in TMEM
-    static constexpr uint32_t SMEM = NL * LAND + MAXK * BSLOT;
+    static constexpr int NL = 4, NM = 3;                     // landing slots; A positions in TMEM
+    static constexpr uint32_t RINGS = NL * LAND + MAXK * BSLOT;
+    static constexpr uint32_t SMEM = RINGS + 8 * kEpiBytes;  // and the drain warps' store blocks
     static constexpr int NTB = 2;                            // accumulator buffers
     static constexpr uint32_t ACOL = NTB * BN;               // first TMEM column of the A parts
     static constexpr uint32_t TMEM_COLS = 512;
@@ -1084,9 +1096,9 @@ __device__ __forceinline__ void tc2kb_split_a_local(const uint8_t* araw, int lro
 // ag.nblk bulk copies of its contiguous blocks (in A's stored order) instead of one TMA box, and the
 // converters read row r's entries at ag.lrow[r] + ag.lk[j] of the slot.
 template <int BN, bool GA>
-__global__ void __launch_bounds__(TC2_THREADS, 1)
+__global__ void __launch_bounds__(TC2_THREADS2, 1)
     k_gemm_tc2kb(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
-                 float* __restrict__ C, int64_t c_is, int N2, int K2, int tiles, int64_t n_items, int a_div,
+                 const __grid_constant__ CUtensorMap mapC, int K2, int tiles, int64_t n_items, int a_div,
                  long long limit, int* err, const float2* __restrict__ ga_base, int64_t ga_is, int ga_mb,
                  const __grid_constant__ AGather ag) {
     // persistent over (item, m tile) jobs: job = blockIdx.x + t * gridDim.x; B' of every k-stage is
@@ -1102,6 +1114,7 @@ __global__ void __launch_bounds__(TC2_THREADS, 1)
     __shared__ uint64_t full[NL], lfree[NL], mfull[NM], mfree[NM], tfull[NTB], tempty[NTB], drain[2], bready;
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
+    __shared__ int conv_seen[2][4];  // per converter group and warp: the last A stage whose slots it saw ready
     __shared__ int16_t s_lrow[GA ? 128 : 1], s_lk[GA ? 16 : 1];  // GA: the slot offsets of rows / K entries
     if (*(volatile const int*)err) return;
     uint8_t* base = (uint8_t*)(((uintptr_t)dyn + 1023) & ~(uintptr_t)1023);
@@ -1137,6 +1150,7 @@ __global__ void __launch_bounds__(TC2_THREADS, 1)
         mbar_init(&drain[0], 1);
         mbar_init(&drain[1], 1);
         mbar_init(&bready, TC2_CONV / 32);
+        for (int w = 0; w < 8; ++w) conv_seen[w >> 2][w & 3] = -1;
         abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -1286,38 +1300,55 @@ __global__ void __launch_bounds__(TC2_THREADS, 1)
         // the MMAs this thread issued finish before TMEM is freed
         tc_commit(&drain[who]);
         mbar_wait_issued(&drain[who], 0);
-    } else if (warp >= 10 && warp <= 13) {
-        // converters: first B' of every stage into its resident slot, then A of every stage into TMEM
-        const int ct = threadIdx.x - 320;
-        int l = 0, m = 0;
+    } else if ((warp >= 10 && warp <= 13) || warp >= 15) {
+        // converters: group 0 (warps 10-13) first builds B' of every stage into its resident slot, then both
+        // groups (warps 15-18 the other) split A into TMEM, alternate stages: one stage's split is a chain of
+        // waits, strided reads (with bank conflicts where A is gathered) and TMEM stores longer than the
+        // stage's share of HBM time.
+        const int grp = warp >= 15 ? 1 : 0, ct = threadIdx.x - 320;
+        int l = 0, m = grp;
         uint32_t lph = 0, mph = 0;
         bool ok = true;
-        for (int s = 0; s < nk; ++s) {
-            const bool go = mbar_wait(&full[l], lph, limit, err) && !*(volatile int*)&abort_flag;
-            if (!__all_sync(0xffffffffu, go)) {
-                atomicExch(&abort_flag, 1);
-                ok = false;
-                break;
+        if (grp == 0) {
+            for (int s = 0; s < nk; ++s) {
+                const bool go = mbar_wait(&full[l], lph, limit, err) && !*(volatile int*)&abort_flag;
+                if (!__all_sync(0xffffffffu, go)) {
+                    atomicExch(&abort_flag, 1);
+                    ok = false;
+                    break;
+                }
+                tc2kb_build_b<BN>(land(l), bslot(s), ct);
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic writes -> tensor core
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(s_addr(&lfree[l])) : "memory");
+                if (++l == NL) {
+                    l = 0;
+                    lph ^= 1u;
+                }
             }
-            tc2kb_build_b<BN>(land(l), bslot(s), ct);
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic writes -> tensor core
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(s_addr(&lfree[l])) : "memory");
-            if (++l == NL) {
-                l = 0;
-                lph ^= 1u;
-            }
+            if (ok && lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(s_addr(&bready)) : "memory");
+        } else {
+            // group 1 starts at A stage 1 (position nk + 1 of the landing sequence), once the B slabs' uses of
+            // the landing slots are over
+            const bool go = mbar_wait(&bready, 0, limit, err) && !*(volatile int*)&abort_flag;
+            ok = __all_sync(0xffffffffu, go);
+            if (!ok) atomicExch(&abort_flag, 1);
+            l = (nk + 1) % NL;
+            lph = (uint32_t)(((nk + 1) / NL) & 1);
         }
-        if (ok && lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(s_addr(&bready)) : "memory");
-        for (int64_t g = 0; g < total && ok; ++g) {
-            // one decision per warp: the TMEM stores of the split are warp-wide (.sync.aligned)
-            const bool go = mbar_wait(&full[l], lph, limit, err) && mbar_wait(&mfree[m], mph ^ 1u, limit, err) &&
+        for (int64_t g = grp; g < total && ok; g += 2) {
+            // one decision per warp: the TMEM stores of the split are warp-wide (.sync.aligned).  As in
+            // k_gemm_tc2, the other group's warp must have seen stage g - 3 first: the slots' uses alternate
+            // between the groups, and a parity alone cannot tell a phase from the one two before.
+            const bool go = (g < 3 || prog_wait(&conv_seen[grp ^ 1][warp & 3], (int)(g - 3), limit, err)) &&
+                            mbar_wait(&full[l], lph, limit, err) && mbar_wait(&mfree[m], mph ^ 1u, limit, err) &&
                             !*(volatile int*)&abort_flag;
             if (!__all_sync(0xffffffffu, go)) {
                 atomicExch(&abort_flag, 1);
                 break;
             }
+            if (lane == 0) prog_set(&conv_seen[grp][warp & 3], (int)g);
             tc_fence_after();  // the MMAs that last read this A position have completed (mfree)
             if (GA)
                 tc2kb_split_a_local(land(l), s_lrow[32 * (warp & 3) + lane], s_lk, tmem, warp & 3, lane,
@@ -1330,12 +1361,14 @@ __global__ void __launch_bounds__(TC2_THREADS, 1)
                 asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(s_addr(&lfree[l])) : "memory");
                 asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(s_addr(&mfull[m])) : "memory");
             }
-            if (++l == NL) {
-                l = 0;
+            l += 2;
+            if (l >= NL) {
+                l -= NL;
                 lph ^= 1u;
             }
-            if (++m == NM) {
-                m = 0;
+            m += 2;
+            if (m >= NM) {
+                m -= NM;
                 mph ^= 1u;
             }
         }
@@ -1360,11 +1393,10 @@ __global__ void __launch_bounds__(TC2_THREADS, 1)
                 }
                 tc_fence_after();
 #pragma unroll
-                for (int c = 0; c < BN / 64; ++c) {
-                    float v[32];
-                    tmem_ld32(tmem + ((uint32_t)(32 * q) << 16) + b * BN + (BN / 2) * half + 32 * c, v);
-#pragma unroll
-                    for (int j = 0; j < 32; ++j) tot[32 * c + j] += v[j];
+                for (int c = 0; c < BN / 32; ++c) {  // 16 columns at a time (registers: 608 threads)
+                    float v[16];
+                    tmem_ld16(tmem + ((uint32_t)(32 * q) << 16) + b * BN + (BN / 2) * half + 16 * c, v);
+                    add_row<16>(tot + 16 * c, v);
                 }
                 tc_fence_before();
                 __syncwarp();
@@ -1375,20 +1407,12 @@ __global__ void __launch_bounds__(TC2_THREADS, 1)
             int64_t item;
             int m0;
             job_of(t, &item, &m0);
-            float* cb = C + item * c_is + (BN / 2) * half + (int64_t)(m0 + 32 * q + ((lane >> 3) << 3)) * N2 +
-                        ((lane & 7) << 2);
+            store_rows<BN / 64>(base + L::RINGS + (warp - 2) * kEpiBytes, &mapC, tot, (BN / 2) * half, m0 + 32 * q,
+                                (int)item, lane);
 #pragma unroll
-            for (int b32 = 0; b32 < BN / 64; ++b32) {
-                float* tt = tot + 32 * b32;
-                transpose_q4(tt, lane);
-#pragma unroll
-                for (int r = 0; r < 8; ++r) {
-                    *(float4*)(cb + (int64_t)r * N2 + 32 * b32) =
-                        make_float4(tt[4 * r], tt[4 * r + 1], tt[4 * r + 2], tt[4 * r + 3]);
-                    tt[4 * r] = tt[4 * r + 1] = tt[4 * r + 2] = tt[4 * r + 3] = 0.f;
-                }
-            }
+            for (int j = 0; j < BN / 2; ++j) tot[j] = 0.f;
         }
+        store_rows_end(lane);
     }
     tc_fence_before();
     __syncthreads();
@@ -1433,6 +1457,25 @@ static bool make_map(CUtensorMap* m, const void* base, int64_t k2, int64_t rows,
     return fn(m, dt, 3, const_cast<void*>(base), dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
               rowb == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+static bool map_raw(CUtensorMap* m, const void* base, int64_t k2, int64_t rows, int64_t items, int64_t item_bytes,
+                    int box_rows) {
+    auto fn = encode_fn();
+    if (!fn) return false;
+    const cuuint64_t dims[3] = {(cuuint64_t)k2, (cuuint64_t)rows, (cuuint64_t)items};
+    const cuuint64_t strides[2] = {(cuuint64_t)(k2 * 4), (cuuint64_t)item_bytes};
+    const cuuint32_t box[3] = {32, (cuuint32_t)box_rows, 1};
+    const cuuint32_t es[3] = {1, 1, 1};
+    return fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void*>(base), dims, strides, box, es,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// C as [items][M][2N] floats, stored in 32 x 32 blocks (store_rows)
+static bool map_c(CUtensorMap* m, const TcArgs& g) {
+    const int64_t M = 1ll << g.mb, N = 1ll << g.nb;
+    return map_raw(m, g.c, 2 * N, M, g.n_items, g.c_is ? g.c_is * 8 : M * N * 8, 32);
 }
 
 // Items of an operand a launch reads: one for an item stride of 0 (the same
@@ -1495,7 +1538,8 @@ static cudaError_t run_gemm_bn(const TcArgs& g, cudaStream_t st) {
         if (!make_map<FORM>(&maps.b[p], (const char*)g.pb + p * pb_part * F::EB, 2 * K, 2 * N,
                             distinct_items(g.b_is, g.b_div, g.n_items), g.pb_is_bytes, BN, ROWB))
             return cudaErrorInvalidValue;
-    const int smem = T::STAGES * (int)T::STAGE_BYTES + 1024;
+    if (!map_c(&maps.c, g)) return cudaErrorInvalidValue;
+    const int smem = T::STAGES * (int)T::STAGE_BYTES + T::EW * T::EBUF * kEpiBytes + 1024;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
@@ -1514,8 +1558,7 @@ static cudaError_t run_gemm_bn(const TcArgs& g, cudaStream_t st) {
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) sms = 152;
     const int64_t jobs = (int64_t)tiles_m * tiles_n * g.n_items;
     const unsigned grid = (unsigned)std::min<int64_t>(jobs, sms);  // persistent: one CTA per SM (shared memory)
-    k_gemm_tc<FORM, BN, ROWB><<<grid, T::THREADS, smem, st>>>(maps, (float*)g.c, g.c_is * 2, (int)M, (int)(2 * N),
-                                                        (int)(2 * K), tiles_n, tiles_m * tiles_n, g.n_items,
+    k_gemm_tc<FORM, BN, ROWB><<<grid, T::THREADS, smem, st>>>(maps, (int)(2 * K), tiles_n, tiles_m * tiles_n, g.n_items,
                                                         g.limit, g.err,
                                                         FORM == TC_FORM_FP16 ? (const float*)g.amax : nullptr,
                                                         item_div(g.a_is, g.a_div), item_div(g.b_is, g.b_div));
@@ -1533,25 +1576,13 @@ static cudaError_t run_gemm(const TcArgs& g, cudaStream_t st) {
     return run_gemm_bn<FORM, 128>(g, st);
 }
 
-static bool map_raw(CUtensorMap* m, const void* base, int64_t k2, int64_t rows, int64_t items, int64_t item_bytes,
-                    int box_rows) {
-    auto fn = encode_fn();
-    if (!fn) return false;
-    const cuuint64_t dims[3] = {(cuuint64_t)k2, (cuuint64_t)rows, (cuuint64_t)items};
-    const cuuint64_t strides[2] = {(cuuint64_t)(k2 * 4), (cuuint64_t)item_bytes};
-    const cuuint32_t box[3] = {32, (cuuint32_t)box_rows, 1};
-    const cuuint32_t es[3] = {1, 1, 1};
-    return fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void*>(base), dims, strides, box, es,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 template <int BN>
 static cudaError_t run_tc2(const TcArgs& g, cudaStream_t st, bool pack2 = false) {
     using L = Tc2<BN>;
     const int64_t M = 1ll << g.mb, N = 1ll << g.nb, K = 1ll << g.kb;
     const bool abc = g.a_is == 0, bbc = g.b_is == 0;
-    CUtensorMap ma, mb;
+    CUtensorMap ma, mb, mc;
+    if (!map_c(&mc, g)) return cudaErrorInvalidValue;
     if (!map_raw(&ma, g.a, 2 * K, M, distinct_items(g.a_is, g.a_div, g.n_items), abc ? M * K * 8 : g.a_is * 8, TC_BM))
         return cudaErrorInvalidValue;
     if (pack2 ? !map_raw(&mb, g.b, 2 * K, N * g.n_items, 1, N * g.n_items * K * 8, BN / 2)
@@ -1582,8 +1613,7 @@ static cudaError_t run_tc2(const TcArgs& g, cudaStream_t st, bool pack2 = false)
     // keep it across the jobs of a CTA
     const int nk = (int)(2 * K / 32);
     const int keep_a = g.a_is && g.a_div > 1 && L::ACOL + 64 * nk <= L::TMEM_COLS;
-    k_gemm_tc2<BN><<<grid, TC2_THREADS2, smem, st>>>(ma, mb, (float*)g.c, g.c_is * 2, (int)M, (int)(2 * N),
-                                                    (int)(2 * K), tiles_n, tiles_m * tiles_n, job_items,
+    k_gemm_tc2<BN><<<grid, TC2_THREADS2, smem, st>>>(ma, mb, mc, (int)(2 * K), tiles_n, tiles_m * tiles_n, job_items,
                                                     item_div(g.a_is, g.a_div), item_div(g.b_is, g.b_div), keep_a,
                                                     pack2 ? 1 : 0, g.limit, g.err);
     return cudaGetLastError();
@@ -1593,7 +1623,8 @@ template <int BN, bool GA>
 static cudaError_t run_tc2kb(const TcArgs& g, cudaStream_t st) {
     using L = Tc2Kb<BN>;
     const int64_t M = 1ll << g.mb, N = 1ll << g.nb, K = 1ll << g.kb;
-    CUtensorMap ma, mb;
+    CUtensorMap ma, mb, mc;
+    if (!map_c(&mc, g)) return cudaErrorInvalidValue;
     memset(&ma, 0, sizeof ma);
     if (!GA && !map_raw(&ma, g.a, 2 * K, M, distinct_items(g.a_is, g.a_div, g.n_items),
                         g.a_is ? g.a_is * 8 : M * K * 8, TC_BM))
@@ -1618,8 +1649,7 @@ static cudaError_t run_tc2kb(const TcArgs& g, cudaStream_t st) {
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) sms = 152;
     const int64_t jobs = (int64_t)tiles * g.n_items;
     const unsigned grid = (unsigned)std::min<int64_t>(jobs, sms);  // one CTA per SM (shared memory)
-    k_gemm_tc2kb<BN, GA><<<grid, TC2_THREADS, smem, st>>>(ma, mb, (float*)g.c, g.c_is * 2, (int)(2 * N),
-                                                          (int)(2 * K), tiles, g.n_items, item_div(g.a_is, g.a_div),
+    k_gemm_tc2kb<BN, GA><<<grid, TC2_THREADS2, smem, st>>>(ma, mb, mc, (int)(2 * K), tiles, g.n_items, item_div(g.a_is, g.a_div),
                                                           g.limit, g.err, g.a, g.a_is, g.mb, g.ag);
     return cudaGetLastError();
 }
@@ -1721,6 +1751,7 @@ cudaError_t launch_tc_gemm(int form, const TcArgs& g, cudaStream_t st) {
 static_assert(TcTile<TC_FORM_3XTF32, 256, 64>::STAGES == 4 && TcTile<TC_FORM_FP16, 256>::STAGES == 4, "stages");
 static_assert(TcTile<TC_FORM_3XTF32, 256, 64>::STAGES * TcTile<TC_FORM_3XTF32, 256, 64>::STAGE_BYTES <= TC_SMEM_LIMIT,
               "smem");
+static_assert(TC_SMEM_LIMIT + 8 * kEpiBytes + 1024 <= 227 * 1024 - 512, "smem");
 static_assert(TcTile<TC_FORM_FP16, 256>::STAGES * TcTile<TC_FORM_FP16, 256>::STAGE_BYTES <= TC_SMEM_LIMIT, "smem");
 static_assert(TcForm<TC_FORM_3XTF32>::STAGES * 4 * TC_BM * TC_ROWB + 1024 <= TC_SMEM_LIMIT + 1024, "smem");
 static_assert(TcForm<TC_FORM_BF16X3>::STAGES * 6 * TC_BM * TC_ROWB + 1024 <= TC_SMEM_LIMIT + 1024, "smem");
