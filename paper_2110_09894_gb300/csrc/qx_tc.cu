@@ -85,73 +85,127 @@ __device__ __forceinline__ float tf32_rna(float x) {
     return __uint_as_float(r);
 }
 
+// The parts of one value: part p of x goes to out[p].
 template <int FORM>
-__device__ __forceinline__ void split(float x, typename TcForm<FORM>::T* out, int64_t part_stride, float scale) {
+__device__ __forceinline__ void split(float x, typename TcForm<FORM>::T* out, float scale) {
     if constexpr (FORM == TC_FORM_FP16) {
         out[0] = __float2half_rn(x * scale);
     } else if constexpr (FORM == TC_FORM_3XTF32) {
         const float hi = tf32_rna(x);
         out[0] = hi;
-        out[part_stride] = x - hi;
+        out[1] = x - hi;
     } else {
         const __nv_bfloat16 b0 = __float2bfloat16_rn(x);
         const float r1 = x - __bfloat162float(b0);
         const __nv_bfloat16 b1 = __float2bfloat16_rn(r1);
         const float r2 = r1 - __bfloat162float(b1);
         out[0] = b0;
-        out[part_stride] = b1;
-        out[2 * part_stride] = __float2bfloat16_rn(r2);
+        out[1] = b1;
+        out[2] = __float2bfloat16_rn(r2);
     }
 }
 
-// A (complex, [R][K] if kmajor else [K][R]) -> parts [P][R][2K]
+// 16 bytes of every part of a run of values x[0 .. n) (n = 16 / sizeof(T)) to o, parts ps elements apart
 template <int FORM>
-__global__ void k_prep_a(const float2* __restrict__ src, int64_t src_is, bool kmajor, typename TcForm<FORM>::T* dst,
-                         int64_t dst_is_elems, int rb, int kb, const float* amax) {
+__device__ __forceinline__ void split_run(const float* x, typename TcForm<FORM>::T* o, int64_t ps, float scale) {
     using T = typename TcForm<FORM>::T;
-    const float sc = amax ? fp16_scale(amax[0]) : 1.f;
-    const int64_t R = (int64_t)1 << rb, K = (int64_t)1 << kb;
-    const int64_t item = blockIdx.y;
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= R * K) return;
-    const int64_t r = idx >> kb, k = idx & (K - 1);
-    const float2 v = src[item * src_is + (kmajor ? idx : k * R + r)];
-    T* o = dst + item * dst_is_elems + r * 2 * K + 2 * k;
-    const int64_t ps = R * 2 * K;
-    split<FORM>(v.x, o, ps, sc);
-    split<FORM>(v.y, o + 1, ps, sc);
+    constexpr int N = 16 / sizeof(T), NP = TcForm<FORM>::NPA;
+    alignas(16) T q[NP][N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        T part[NP];
+        split<FORM>(x[i], part, scale);
+#pragma unroll
+        for (int p = 0; p < NP; ++p) q[p][i] = part[p];
+    }
+#pragma unroll
+    for (int p = 0; p < NP; ++p) *(int4*)(o + p * ps) = *(const int4*)q[p];
 }
 
-// B (complex, [R][K] if kmajor else [K][R]) -> parts [P][2R][2K]:
-// row 2r = (re, -im) per k, row 2r+1 = (im, re)
-template <int FORM>
-__global__ void k_prep_b(const float2* __restrict__ src, int64_t src_is, bool kmajor, typename TcForm<FORM>::T* dst,
-                         int64_t dst_is_elems, int rb, int kb, const float* amax) {
+// Operand split, bound by HBM: every thread takes the complex entries of 16 bytes of a part (2 in TF32, 4
+// in the 16-bit forms) of one row, so that loads and stores are 16 bytes; writing the 16-bit parts one
+// by one ran at 1.9 to 4.4 TB/s.  Both operands, with the FP16 form's maximum (us): FP16 128 x 64 x 64 for
+// 12864 items 1026 -> 495; BF16x3 2048 x 512 x 512 for 87 558 -> 372; 3xTF32 the same for 188 1056 -> 959.
+// An operand stored [K][R] goes through a 32 x 32 tile of shared memory.
+//   A (EXPAND = false): parts [P][R][2K], A's interleaved storage
+//   B (EXPAND = true):  parts [P][2R][2K], row 2r = (re, -im) per k, row 2r + 1 = (im, re)
+template <int FORM, bool EXPAND>
+__global__ void __launch_bounds__(256) k_prep(const float2* __restrict__ src, int64_t src_is, bool kmajor,
+                                              typename TcForm<FORM>::T* dst, int64_t dst_is_elems, int rb, int kb,
+                                              const float* amax) {
     using T = typename TcForm<FORM>::T;
-    const float sc = amax ? fp16_scale(amax[1]) : 1.f;
+    constexpr int V = 8 / sizeof(T), VB = V == 4 ? 2 : 1;  // complex entries per thread, log2
+    const float sc = amax ? fp16_scale(amax[EXPAND ? 1 : 0]) : 1.f;
     const int64_t R = (int64_t)1 << rb, K = (int64_t)1 << kb;
-    const int64_t item = blockIdx.y;
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= R * K) return;
-    const int64_t r = idx >> kb, k = idx & (K - 1);
-    const float2 v = src[item * src_is + (kmajor ? idx : k * R + r)];
-    T* o = dst + item * dst_is_elems + (2 * r) * 2 * K + 2 * k;
-    const int64_t ps = 4 * R * K;
-    split<FORM>(v.x, o, ps, sc);
-    split<FORM>(-v.y, o + 1, ps, sc);
-    split<FORM>(v.y, o + 2 * K, ps, sc);
-    split<FORM>(v.x, o + 2 * K + 1, ps, sc);
+    src += (int64_t)blockIdx.y * src_is;
+    dst += (int64_t)blockIdx.y * dst_is_elems;
+    auto put = [&](const float2* v, int64_t r, int64_t k) {
+        float x[2 * V];
+        const int64_t ps = (EXPAND ? 4 : 2) * R * K;
+        T* o = dst + (EXPAND ? 2 * r : r) * 2 * K + 2 * k;
+#pragma unroll
+        for (int i = 0; i < V; ++i) {
+            x[2 * i] = v[i].x;
+            x[2 * i + 1] = EXPAND ? -v[i].y : v[i].y;
+        }
+        split_run<FORM>(x, o, ps, sc);
+        if constexpr (EXPAND) {
+#pragma unroll
+            for (int i = 0; i < V; ++i) {
+                x[2 * i] = v[i].y;
+                x[2 * i + 1] = v[i].x;
+            }
+            split_run<FORM>(x, o + 2 * K, ps, sc);
+        }
+    };
+    float2 v[V];
+    if (kmajor) {
+        const int64_t idx = ((int64_t)blockIdx.x * 256 + threadIdx.x) << VB;
+        if (idx >= R * K) return;
+#pragma unroll
+        for (int i = 0; i < V; i += 2) {
+            const float4 q = *(const float4*)(src + idx + i);
+            v[i] = make_float2(q.x, q.y);
+            v[i + 1] = make_float2(q.z, q.w);
+        }
+        put(v, idx >> kb, idx & (K - 1));
+        return;
+    }
+    // 32 rows x 32 k per block (R, K >= 32)
+    __shared__ float2 tile[32][33];
+    const int64_t rt = R >> 5, r0 = (blockIdx.x % rt) << 5, k0 = (blockIdx.x / rt) << 5;
+    for (int i = threadIdx.x; i < 1024; i += 256) tile[i >> 5][i & 31] = src[(k0 + (i >> 5)) * R + r0 + (i & 31)];
+    __syncthreads();
+    for (int i = threadIdx.x; i < 1024 >> VB; i += 256) {
+        const int k = (i & ((32 >> VB) - 1)) << VB, r = i >> (5 - VB);
+#pragma unroll
+        for (int j = 0; j < V; ++j) v[j] = tile[k + j][r];
+        put(v, r0 + r, k0 + k);
+    }
+}
+template <int FORM, bool EXPAND>
+static cudaError_t prep(const float2* src, int64_t src_is, bool kmajor, void* dst, int64_t dst_is_bytes, int rb, int kb,
+                        int64_t items, const float* amax, cudaStream_t st) {
+    using T = typename TcForm<FORM>::T;
+    const int64_t entries = (int64_t)1 << (rb + kb);
+    const int64_t blocks = kmajor ? (entries * (int64_t)sizeof(T) / 8 + 255) / 256 : entries >> 10;
+    const dim3 grid((unsigned)blocks, (unsigned)items);
+    k_prep<FORM, EXPAND><<<grid, 256, 0, st>>>(src, src_is, kmajor, (T*)dst, dst_is_bytes / (int64_t)sizeof(T), rb, kb,
+                                               amax);
+    return cudaGetLastError();
 }
 
-// max |re|, |im| over an operand (all items); non-negative floats order like their bit patterns
-__global__ void k_absmax(const float2* __restrict__ src, int64_t src_is, int64_t per_item, int64_t n_items,
-                         float* out) {
+// max |re|, |im| over an operand of 2^eb entries per item (all items); non-negative floats order like their
+// bit patterns
+__global__ void __launch_bounds__(256) k_absmax(const float2* __restrict__ src, int64_t src_is, int eb, int64_t n_items,
+                                                float* out) {
     float m = 0.f;
-    const int64_t total = per_item * n_items;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t item = i / per_item, e = i - item * per_item;
-        const float2 v = src[item * src_is + e];
-        m = fmaxf(m, fmaxf(fabsf(v.x), fabsf(v.y)));
+    const int64_t total = n_items << (eb - 1), step = (int64_t)gridDim.x * 256;  // pairs of entries
+#pragma unroll 4
+    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < total; i += step) {
+        const int64_t item = i >> (eb - 1), e = i & (((int64_t)1 << (eb - 1)) - 1);
+        const float4 v = *(const float4*)(src + item * src_is + 2 * e);
+        m = fmaxf(m, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
     }
     for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
     if ((threadIdx.x & 31) == 0) atomicMax((unsigned int*)out, __float_as_uint(m));
@@ -1495,8 +1549,6 @@ int tc_products(int form) { return form == TC_FORM_3XTF32 ? 3 : form == TC_FORM_
 
 template <int FORM>
 static cudaError_t run_prep(const TcArgs& g, cudaStream_t st) {
-    using F = TcForm<FORM>;
-    using T = typename F::T;
     const int64_t M = 1ll << g.mb, N = 1ll << g.nb, K = 1ll << g.kb;
     const float* amax = nullptr;
     if constexpr (FORM == TC_FORM_FP16) {
@@ -1504,22 +1556,19 @@ static cudaError_t run_prep(const TcArgs& g, cudaStream_t st) {
         cudaError_t e = cudaMemsetAsync(g.amax, 0, 2 * sizeof(float), st);
         if (e != cudaSuccess) return e;
         const int64_t na = distinct_items(g.a_is, g.a_div, g.n_items), nb_ = distinct_items(g.b_is, g.b_div, g.n_items);
-        k_absmax<<<(unsigned)std::min<int64_t>((M * K * na + 255) / 256, 4096), 256, 0, st>>>(g.a, g.a_is, M * K, na,
-                                                                                               g.amax);
-        k_absmax<<<(unsigned)std::min<int64_t>((N * K * nb_ + 255) / 256, 4096), 256, 0, st>>>(g.b, g.b_is, N * K,
-                                                                                                nb_, g.amax + 1);
+        auto blocks = [](int64_t entries) { return (unsigned)std::min<int64_t>((entries / 2 + 255) / 256, 152 * 8); };
+        k_absmax<<<blocks(M * K * na), 256, 0, st>>>(g.a, g.a_is, g.mb + g.kb, na, g.amax);
+        k_absmax<<<blocks(N * K * nb_), 256, 0, st>>>(g.b, g.b_is, g.nb + g.kb, nb_, g.amax + 1);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         amax = g.amax;
     }
     // each distinct operand item is split once
-    dim3 grid((unsigned)((M * K + 255) / 256), (unsigned)distinct_items(g.a_is, g.a_div, g.n_items));
-    k_prep_a<FORM><<<grid, 256, 0, st>>>(g.a, g.a_is, g.a_kmajor, (T*)g.pa, g.pa_is_bytes / F::EB, g.mb, g.kb, amax);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = prep<FORM, false>(g.a, g.a_is, g.a_kmajor, g.pa, g.pa_is_bytes, g.mb, g.kb,
+                                      distinct_items(g.a_is, g.a_div, g.n_items), amax, st);
     if (e != cudaSuccess) return e;
-    dim3 grid2((unsigned)((N * K + 255) / 256), (unsigned)distinct_items(g.b_is, g.b_div, g.n_items));
-    k_prep_b<FORM><<<grid2, 256, 0, st>>>(g.b, g.b_is, g.b_kmajor, (T*)g.pb, g.pb_is_bytes / F::EB, g.nb, g.kb, amax);
-    return cudaGetLastError();
+    return prep<FORM, true>(g.b, g.b_is, g.b_kmajor, g.pb, g.pb_is_bytes, g.nb, g.kb,
+                            distinct_items(g.b_is, g.b_div, g.n_items), amax, st);
 }
 
 template <int FORM, int BN, int ROWB = TC_ROWB>
