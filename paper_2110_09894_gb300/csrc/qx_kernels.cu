@@ -1135,7 +1135,7 @@ __global__ void __launch_bounds__(256) k_dot_c64(const float2* __restrict__ A, i
 // C = sum_k A[k] B[p(k)], B read through the permutation's tiles (as k_permute: a tile in input
 // order into shared memory, then walked in A's order), so the permuted copy of B never goes to HBM.
 // One CTA per pair; per-thread FP32 partials, then a fixed-order tree.
-__global__ void __launch_bounds__(256) k_dot_perm(const PermDesc d, const PermTables tb, const ItemCtx ic,
+__global__ void __launch_bounds__(256, 4) k_dot_perm(const PermDesc d, const PermTables tb, const ItemCtx ic,
                                                   const float2* __restrict__ A, int64_t a_is, float2* __restrict__ C,
                                                   int64_t c_is, int a_div) {
     constexpr int LO = kPermLoBits, LM = (1 << LO) - 1;
@@ -1168,22 +1168,48 @@ __global__ void __launch_bounds__(256) k_dot_perm(const PermDesc d, const PermTa
             ob += tb.outer_out[i];
             u &= u - 1;
         }
-        for (int j = tid; j < n; j += 256) tile[pad32(j)] = d.in.base[ib + s_in[j & LM] + s_in[64 + (j >> LO)]];
+        // B's loads all in flight, then A's while B's entries settle in shared memory
+        float2 v[kPermPer];
+#pragma unroll
+        for (int k = 0; k < kPermPer; ++k) {
+            const int j = tid + 256 * k;
+            if (j < n) v[k] = d.in.base[ib + s_in[j & LM] + s_in[64 + (j >> LO)]];
+        }
+#pragma unroll
+        for (int k = 0; k < kPermPer; ++k) {
+            const int j = tid + 256 * k;
+            if (j < n) tile[pad32(j)] = v[k];
+        }
+#pragma unroll
+        for (int k = 0; k < kPermPer; ++k) {
+            const int j = tid + 256 * k;
+            if (j < n) v[k] = Ap[ob + s_out[j & LM] + s_out[64 + (j >> LO)]];
+        }
         __syncthreads();
-        for (int j = tid; j < n; j += 256)
-            cfma(acc, Ap[ob + s_out[j & LM] + s_out[64 + (j >> LO)]], tile[pad32(s_map[j & LM] | s_map[64 + (j >> LO)])]);
+#pragma unroll
+        for (int k = 0; k < kPermPer; ++k) {
+            const int j = tid + 256 * k;
+            if (j < n) cfma(acc, v[k], tile[pad32(s_map[j & LM] | s_map[64 + (j >> LO)])]);
+        }
         __syncthreads();
     }
     red[tid] = acc;
     __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
+    for (int w = 128; w > 16; w >>= 1) {
         if (tid < w) {
             red[tid].x += red[tid + w].x;
             red[tid].y += red[tid + w].y;
         }
         __syncthreads();
     }
-    if (tid == 0) C[item * c_is] = red[0];
+    if (tid < 32) {
+        float2 x = red[tid];
+        for (int w = 16; w > 0; w >>= 1) {  // the same tree within a warp
+            x.x += __shfl_down_sync(0xffffffffu, x.x, w);
+            x.y += __shfl_down_sync(0xffffffffu, x.y, w);
+        }
+        if (tid == 0) C[item * c_is] = x;
+    }
 }
 
 cudaError_t launch_dot_perm(const PermDesc& d, const ItemCtx& ic, int64_t n_items, const float2* a, int64_t a_is,
