@@ -91,9 +91,9 @@ struct Op {
     int dst = -1;           // output storage
     int tc = 0;             // tensor-core form (0: SIMT)
     int spa = -1, spb = -1; // split-part storages of the tensor-core form
-    // direct 3xTF32 step on the resident-B' kernel that reads A where it is stored (no permute): address
+    // direct 3xTF32 step that reads A where it is stored (no permute): address
     // position of each row bit and of each complex K bit of A
-    bool a_gather = false;
+    int a_gather = 0;       // 1: on the resident-B' kernel in blocks of at least 2^8 entries, 2: otherwise
     std::vector<int8_t> ag_mpos, ag_kpos;
     double flops = 0;
 };
@@ -978,14 +978,17 @@ static int compile_plan(qx_ctx* h, const int64_t* order, int64_t n_steps, const 
             c.cost = (c.pa ? (double)node_entries(GA) : 0.0) + (c.pb ? (double)node_entries(GB) : 0.0);
             if (best.cost < 0 || c.cost < best.cost) best = c;
         }
-        // The resident-B' direct kernel (B invariant and one tile wide, every K stage of B' resident, A
-        // per item; the conditions of tc2_resident_b) gathers A where it is stored, row and K bits at
-        // their positions, instead of reading a copy permuted to K-major: the permute is left out.
-        // The stage tile must be a few contiguous blocks of A (agather_tile).
-        const int fa_n = (int)fA.size(), fb_n = (int)fB.size();
-        const bool kb_fits = (fb_n == 6 && kb <= 6) || (fb_n == 5 && kb <= 7);
-        bool a_gather = direct && best.pa && kb_fits && GB.level == 0 && GA.level == level && !GA.leaf &&
-                        GA.fix.empty() && fa_n + kb == (int)GA.legs.size() && fa_n <= kMaxRank;
+        // The direct kernels gather an A of their own level where it is stored, row and K bits at their
+        // positions, instead of reading a copy permuted to K-major: the permute (16 bytes an entry through
+        // HBM) is left out.  The stage tile must be a few contiguous blocks of A (agather_tile: one bulk copy
+        // per lane of the producer warp, 512 bytes each at least).  B at most two column tiles wide: every
+        // column tile converts A's tile again, out of a slot whose banks conflict where the K bits are low
+        // ones.  Measured, GEMM + permute before and GEMM alone after: one tile, m=14 k=6 n=6 per pair
+        // 1225 + 1000 -> 1320 us (1024 items); two tiles, m=11 k=5 n=7 200 -> 152 us (300 items); four
+        // tiles, m=8 k=12 n=8 3575 + 1030 -> 5250 us, so that one keeps its permute.
+        const int fa_n = (int)fA.size();
+        int a_gather = direct && fB.size() <= 7 && best.pa && GA.level == level && !GA.leaf && GA.fix.empty() &&
+                       fa_n + kb == (int)GA.legs.size() && fa_n <= kMaxRank && kb <= 16;
         std::vector<int8_t> ag_m, ag_k;
         if (a_gather) {
             auto pos_of = [&](int leg) {
@@ -996,7 +999,9 @@ static int compile_plan(qx_ctx* h, const int64_t* order, int64_t n_steps, const 
             AGather probe{};
             for (int i = 0; i < fa_n; ++i) probe.mpos[i] = ag_m[i];
             for (int i = 0; i < kb; ++i) probe.kpos[i] = ag_k[i];
-            a_gather = agather_tile(&probe, fa_n, kb);
+            const int fb_n = (int)fB.size();
+            const bool resident = GB.level == 0 && ((fb_n == 6 && kb <= 6) || (fb_n == 5 && kb <= 7));
+            a_gather = !agather_tile(&probe, fa_n, kb) ? 0 : resident && probe.run >= 8 ? 1 : 2;
         }
         if (a_gather) {
             best.pa = false;
@@ -1024,7 +1029,7 @@ static int compile_plan(qx_ctx* h, const int64_t* order, int64_t n_steps, const 
         g.a_km = best.akm;
         g.b_km = best.bkm;
         if (a_gather) {
-            g.a_gather = true;
+            g.a_gather = a_gather;
             g.ag_mpos = ag_m;
             g.ag_kpos = ag_k;
         }
@@ -2814,7 +2819,7 @@ int qx_describe_plan(qx_handle h, char* buf, int64_t len, int64_t* needed) {
             snprintf(line, sizeof line,
                      "%zu step=%lld %s %s m=%d k=%d n=%d a_kmajor=%d b_kmajor=%d scatter=%d a_gather=%d\n", i,
                      (long long)op.step, kind, op.level == 2 ? "pair" : op.level == 1 ? "slice" : "shared", op.mb, op.kb,
-                     op.nb, (int)op.a_km, (int)op.b_km, (int)!op.out_pos.empty(), (int)op.a_gather);
+                     op.nb, (int)op.a_km, (int)op.b_km, (int)!op.out_pos.empty(), op.a_gather);
         }
         out += line;
         if (op.type == OP_SMALL) {  // address positions in X of the contracted legs

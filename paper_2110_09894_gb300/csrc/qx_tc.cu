@@ -696,9 +696,10 @@ __device__ __forceinline__ void split4(float4 v, float4& hi, float4& lo) {
 // Convert a landed slab pair (`land`) into an MMA slot (`ms`, TMEM columns ahi / ahi + 32) with the
 // converter warps: thread (quarter qq, lane) splits row 32 qq + lane of A into TMEM (row = lane),
 // then the threads ct = 0 .. TC2_CONV - 1 build B' hi / lo in shared memory.
-template <int BN>
+// GA (A gathered in place): row r's 16 K entries sit at entries lrow + lk[j] of the slot.
+template <int BN, bool GA>
 __device__ __forceinline__ void tc2_convert(const uint8_t* land, uint8_t* ms, int ct, uint32_t tmem, int qq,
-                                            int lane, uint32_t ahi, bool with_a) {
+                                            int lane, uint32_t ahi, bool with_a, int lrow, const int16_t* lk) {
     using L = Tc2<BN>;
     const int r = 32 * qq + lane;
     const uint32_t lanes = (uint32_t)(32 * qq) << 16;
@@ -708,7 +709,15 @@ __device__ __forceinline__ void tc2_convert(const uint8_t* land, uint8_t* ms, in
     float4 va[8], vb[NBC];
     if (with_a) {
 #pragma unroll
-        for (int j = 0; j < 8; ++j) va[j] = *(const float4*)(land + r * 128 + ((j ^ (r & 7)) << 4));
+        for (int j = 0; j < 8; ++j) {
+            if (GA) {
+                const float2 x = *(const float2*)(land + 8 * (lrow + lk[2 * j]));
+                const float2 y = *(const float2*)(land + 8 * (lrow + lk[2 * j + 1]));
+                va[j] = make_float4(x.x, x.y, y.x, y.y);
+            } else {
+                va[j] = *(const float4*)(land + r * 128 + ((j ^ (r & 7)) << 4));
+            }
+        }
     }
 #pragma unroll
     for (int i = 0; i < NBC; ++i) {
@@ -749,11 +758,35 @@ __device__ __forceinline__ void tc2_convert(const uint8_t* land, uint8_t* ms, in
     asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
 
-template <int BN>
+// bulk copy of `bytes` (a multiple of 16, both addresses 16-byte aligned) into shared memory, completing
+// on an mbarrier's transaction count
+__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                     s_addr(dst)),
+                 "l"(src), "r"(bytes), "r"(s_addr(bar))
+                 : "memory");
+}
+
+// A gathered in place (AGather): base address offset of a job's tile (its item's entries and row bits 7 and
+// up), and of its K stage (K bits 4 and up)
+__device__ __forceinline__ int64_t gather_rows(const AGather& ag, int64_t item_off, int m0, int mb) {
+    for (int b = 7; b < mb; ++b)
+        if ((m0 >> b) & 1) item_off += (int64_t)1 << ag.mpos[b];
+    return item_off;
+}
+__device__ __forceinline__ int64_t gather_stage(const AGather& ag, int it) {
+    int64_t o = 0;
+    for (int b = 0; (it >> b) > 0; ++b)
+        if ((it >> b) & 1) o += (int64_t)1 << ag.kpos[4 + b];
+    return o;
+}
+
+template <int BN, bool GA>
 __global__ void __launch_bounds__(TC2_THREADS2, 1)
     k_gemm_tc2(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
                const __grid_constant__ CUtensorMap mapC, int K2, int tiles_n, int tiles, int64_t n_items,
-               int a_div, int b_div, int keep_a, int pack2, long long limit, int* err) {
+               int a_div, int b_div, int keep_a, int pack2, long long limit, int* err,
+               const float2* __restrict__ ga_base, int64_t ga_is, int ga_mb, const __grid_constant__ AGather ag) {
     // persistent over (pair, tile) jobs: job = blockIdx.x + t * gridDim.x; the
     // k-stages of successive jobs form one sequence g = t * nk + it, so both
     // rings stay full across tile boundaries.
@@ -764,6 +797,9 @@ __global__ void __launch_bounds__(TC2_THREADS2, 1)
     // pack2 (N = BN / 4 complex per item, B dense per item, both items of a job on the same A): a job
     // covers items 2 i and 2 i + 1 side by side, B's rows of both come in one TMA box (B read as one
     // [items x N][2K] matrix), and drain half h writes item 2 i + h.
+    // GA (never with keep_a or pack2): the lanes of the producer warp bring a stage's 128 x 16 tile of A
+    // where it is stored, one bulk copy of a contiguous block each, instead of one TMA box of a copy that
+    // a permute would have to write first.
     using L = Tc2<BN>;
     constexpr int BK = 32;  // TF32 elements per stage (one 128-byte slab)
     constexpr int NL = L::NL, NM = L::NM, NTB = L::NTB;
@@ -773,6 +809,7 @@ __global__ void __launch_bounds__(TC2_THREADS2, 1)
     __shared__ uint64_t full[NL], lfree[NL], mfull[NM], mfree[NM], tfull[NTB], tempty[NTB], drain[2];
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
+    __shared__ int16_t s_lrow[GA ? 128 : 1], s_lk[GA ? 16 : 1];  // GA: the slot offsets of rows / K entries
     __shared__ int conv_seen[2][4];  // per converter group and warp: the last stage whose slots it saw ready
     if (*(volatile const int*)err) return;
     uint8_t* base = (uint8_t*)(((uintptr_t)dyn + 1023) & ~(uintptr_t)1023);
@@ -792,6 +829,10 @@ __global__ void __launch_bounds__(TC2_THREADS2, 1)
         *n0 = (tile % tiles_n) * BN;  // row of B'; raw B row n0 / 2
         *akey = (*item / a_div) * (tiles / tiles_n) + tile / tiles_n;
     };
+    if (GA) {
+        if (threadIdx.x < 128) s_lrow[threadIdx.x] = ag.lrow[threadIdx.x];
+        if (threadIdx.x < 16) s_lk[threadIdx.x] = ag.lk[threadIdx.x];
+    }
     // Every role walks the stages g = 0, 1, ... with counters (ring slot and its phase, stage within
     // the job, job) advanced by one step at a time: 64-bit divisions per stage would cost more
     // cycles than a stage's MMAs.  A job is decoded (job_of) once, at its first or last stage.
@@ -825,7 +866,42 @@ __global__ void __launch_bounds__(TC2_THREADS2, 1)
     tc_fence_after();
     const uint32_t tmem = tmem_slot;
 
-    if (warp == 0 && lane == 0) {
+    if (GA && warp == 0) {
+        int64_t issued = 0, t = 0, item = 0, akey = 0, rowb = 0;
+        int l = 0, it = 0, m0 = 0, n0 = 0;
+        uint32_t lph = 0;
+        const uint32_t blk_bytes = 8u << ag.run;
+        const int64_t my_blk = lane < ag.nblk ? ag.blk_off[lane] : 0;
+        for (int64_t g = 0; g < total; ++g) {
+            const bool go = mbar_wait(&lfree[l], lph ^ 1u, limit, err) && !*(volatile int*)&abort_flag;
+            if (!__all_sync(0xffffffffu, go)) {
+                atomicExch(&abort_flag, 1);
+                break;
+            }
+            if (it == 0) {
+                job_of(t, &item, &m0, &n0, &akey);
+                rowb = gather_rows(ag, (item / a_div) * ga_is, m0, ga_mb);
+            }
+            if (lane == 0) mbar_expect_tx(&full[l], L::LAND);
+            __syncwarp();
+            if (lane < ag.nblk)
+                bulk_load(land(l) + (size_t)lane * blk_bytes, ga_base + rowb + gather_stage(ag, it) + my_blk, blk_bytes,
+                          &full[l]);
+            if (lane == 0) tma_load_3d(land(l) + L::A, &mapB, it * BK, n0 >> 1, (int)(item / b_div), &full[l]);
+            ++issued;
+            if (++it == nk) {
+                it = 0;
+                ++t;
+            }
+            if (++l == NL) {
+                l = 0;
+                lph ^= 1u;
+            }
+        }
+        // the copies in flight land before the CTA exits (immediate unless a wait gave up)
+        for (int64_t g = (issued > NL ? issued - NL : 0); g < issued; ++g)
+            mbar_wait_issued(&full[g % NL], (uint32_t)((g / NL) & 1));
+    } else if (!GA && warp == 0 && lane == 0) {
         int64_t issued = 0, t = 0, item = 0, akey = 0, prev_key = -1;
         int l = 0, it = 0, m0 = 0, n0 = 0, ia = 0, ib = 0;
         uint32_t lph = 0;
@@ -956,8 +1032,8 @@ __global__ void __launch_bounds__(TC2_THREADS2, 1)
                 }
             }
             tc_fence_after();  // the MMAs that last read this MMA slot have completed (mfree)
-            tc2_convert<BN>(land(l), mslot(m), ct, tmem, warp & 3, lane,
-                            L::ACOL + 64 * (uint32_t)(keep_a ? it : m), with_a);
+            tc2_convert<BN, GA>(land(l), mslot(m), ct, tmem, warp & 3, lane, L::ACOL + 64 * (uint32_t)(keep_a ? it : m),
+                                with_a, GA ? s_lrow[32 * (warp & 3) + lane] : 0, s_lk);
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic writes -> tensor core
             tc_fence_before();
             __syncwarp();
@@ -1113,15 +1189,6 @@ __device__ __forceinline__ void tc2kb_split_a(const uint8_t* araw, uint32_t tmem
     asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
 
-// bulk copy of `bytes` (a multiple of 16, both addresses 16-byte aligned) into shared memory, completing
-// on an mbarrier's transaction count
-__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                     s_addr(dst)),
-                 "l"(src), "r"(bytes), "r"(s_addr(bar))
-                 : "memory");
-}
-
 // A hi / lo of one gathered slab (GA): row r's 16 K entries sit at entries lrow + lk[j] of the slot
 __device__ __forceinline__ void tc2kb_split_a_local(const uint8_t* araw, int lrow, const int16_t* lk, uint32_t tmem,
                                                     int qq, int lane, uint32_t ahi) {
@@ -1219,44 +1286,47 @@ __global__ void __launch_bounds__(TC2_THREADS2, 1)
     tc_fence_after();
     const uint32_t tmem = tmem_slot;
 
-    if (GA && warp == 0 && lane == 0) {
+    if (GA && warp == 0) {
         int64_t issued = 0, t = 0, item = 0;
         int l = 0, it = 0, m0 = 0;
         uint32_t lph = 0;
         bool ok = true;
         for (int s = 0; s < nk && ok; ++s) {  // the raw B slab of every stage (TMA)
-            if (!mbar_wait(&lfree[l], lph ^ 1u, limit, err) || *(volatile int*)&abort_flag) {
+            const bool go = mbar_wait(&lfree[l], lph ^ 1u, limit, err) && !*(volatile int*)&abort_flag;
+            if (!__all_sync(0xffffffffu, go)) {
                 atomicExch(&abort_flag, 1);
                 ok = false;
                 break;
             }
-            mbar_expect_tx(&full[l], L::BRAW);
-            tma_load_3d(land(l), &mapB, s * BK, 0, 0, &full[l]);
+            if (lane == 0) {
+                mbar_expect_tx(&full[l], L::BRAW);
+                tma_load_3d(land(l), &mapB, s * BK, 0, 0, &full[l]);
+            }
             ++issued;
             if (++l == NL) {
                 l = 0;
                 lph ^= 1u;
             }
         }
+        // one block of a stage's tile per lane (see k_gemm_tc2)
         const uint32_t blk_bytes = 8u << ag.run;
+        const int64_t my_blk = lane < ag.nblk ? ag.blk_off[lane] : 0;
         int64_t rowb = 0;
         for (int64_t g = 0; g < total && ok; ++g) {
-            if (!mbar_wait(&lfree[l], lph ^ 1u, limit, err) || *(volatile int*)&abort_flag) {
+            const bool go = mbar_wait(&lfree[l], lph ^ 1u, limit, err) && !*(volatile int*)&abort_flag;
+            if (!__all_sync(0xffffffffu, go)) {
                 atomicExch(&abort_flag, 1);
                 break;
             }
-            if (it == 0) {  // the job's tile base in A: its item and row bits 7 and up
+            if (it == 0) {
                 job_of(t, &item, &m0);
-                rowb = (item / a_div) * ga_is;
-                for (int b = 7; b < ga_mb; ++b)
-                    if ((m0 >> b) & 1) rowb += (int64_t)1 << ag.mpos[b];
+                rowb = gather_rows(ag, (item / a_div) * ga_is, m0, ga_mb);
             }
-            int64_t tb = rowb;  // and the stage's K bits 4 and up
-            for (int b = 0; (it >> b) > 0; ++b)
-                if ((it >> b) & 1) tb += (int64_t)1 << ag.kpos[4 + b];
-            mbar_expect_tx(&full[l], L::A);
-            for (int b = 0; b < ag.nblk; ++b)
-                bulk_load(land(l) + (size_t)b * blk_bytes, ga_base + tb + ag.blk_off[b], blk_bytes, &full[l]);
+            if (lane == 0) mbar_expect_tx(&full[l], L::A);
+            __syncwarp();
+            if (lane < ag.nblk)
+                bulk_load(land(l) + (size_t)lane * blk_bytes, ga_base + rowb + gather_stage(ag, it) + my_blk, blk_bytes,
+                          &full[l]);
             ++issued;
             if (++it == nk) {
                 it = 0;
@@ -1625,14 +1695,16 @@ static cudaError_t run_gemm(const TcArgs& g, cudaStream_t st) {
     return run_gemm_bn<FORM, 128>(g, st);
 }
 
-template <int BN>
+template <int BN, bool GA>
 static cudaError_t run_tc2(const TcArgs& g, cudaStream_t st, bool pack2 = false) {
     using L = Tc2<BN>;
     const int64_t M = 1ll << g.mb, N = 1ll << g.nb, K = 1ll << g.kb;
     const bool abc = g.a_is == 0, bbc = g.b_is == 0;
     CUtensorMap ma, mb, mc;
     if (!map_c(&mc, g)) return cudaErrorInvalidValue;
-    if (!map_raw(&ma, g.a, 2 * K, M, distinct_items(g.a_is, g.a_div, g.n_items), abc ? M * K * 8 : g.a_is * 8, TC_BM))
+    memset(&ma, 0, sizeof ma);
+    if (!GA && !map_raw(&ma, g.a, 2 * K, M, distinct_items(g.a_is, g.a_div, g.n_items), abc ? M * K * 8 : g.a_is * 8,
+                        TC_BM))
         return cudaErrorInvalidValue;
     if (pack2 ? !map_raw(&mb, g.b, 2 * K, N * g.n_items, 1, N * g.n_items * K * 8, BN / 2)
               : !map_raw(&mb, g.b, 2 * K, N, distinct_items(g.b_is, g.b_div, g.n_items), bbc ? N * K * 8 : g.b_is * 8,
@@ -1647,7 +1719,7 @@ static cudaError_t run_tc2(const TcArgs& g, cudaStream_t st, bool pack2 = false)
     {
         std::lock_guard<std::mutex> lk(mu);
         if (dev < 256 && !((done[dev >> 6] >> (dev & 63)) & 1)) {
-            e = cudaFuncSetAttribute(k_gemm_tc2<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+            e = cudaFuncSetAttribute(k_gemm_tc2<BN, GA>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
             if (e != cudaSuccess) return e;
             done[dev >> 6] |= 1ull << (dev & 63);
         }
@@ -1661,10 +1733,10 @@ static cudaError_t run_tc2(const TcArgs& g, cudaStream_t st, bool pack2 = false)
     // A shared by the items of a slice, and all of its k-stages fit in TMEM after the accumulators:
     // keep it across the jobs of a CTA
     const int nk = (int)(2 * K / 32);
-    const int keep_a = g.a_is && g.a_div > 1 && L::ACOL + 64 * nk <= L::TMEM_COLS;
-    k_gemm_tc2<BN><<<grid, TC2_THREADS2, smem, st>>>(ma, mb, mc, (int)(2 * K), tiles_n, tiles_m * tiles_n, job_items,
+    const int keep_a = !GA && g.a_is && g.a_div > 1 && L::ACOL + 64 * nk <= L::TMEM_COLS;
+    k_gemm_tc2<BN, GA><<<grid, TC2_THREADS2, smem, st>>>(ma, mb, mc, (int)(2 * K), tiles_n, tiles_m * tiles_n, job_items,
                                                     item_div(g.a_is, g.a_div), item_div(g.b_is, g.b_div), keep_a,
-                                                    pack2 ? 1 : 0, g.limit, g.err);
+                                                    pack2 ? 1 : 0, g.limit, g.err, g.a, g.a_is, g.mb, g.ag);
     return cudaGetLastError();
 }
 
@@ -1713,7 +1785,7 @@ bool agather_tile(AGather* g, int mb, int kb) {
     std::sort(sorted, sorted + 11);
     int run = 0;
     while (run < 11 && sorted[run] == run) ++run;
-    if (run < 8) return false;
+    if (run < 6) return false;
     // local position of a tile bit: its own below run, else run + its rank among the others
     int local[11];
     for (int i = 0; i < 11; ++i) {
@@ -1751,19 +1823,20 @@ bool agather_tile(AGather* g, int mb, int kb) {
 cudaError_t launch_tc2_gemm(const TcArgs& g, cudaStream_t st) {
     if (!(g.mb >= 7 && g.nb >= 5 && g.kb >= 4 && g.n_items > 0 && g.n_items <= 65535)) return cudaErrorInvalidValue;
     if ((!g.a_kmajor && !g.ag.on) || !g.b_kmajor) return cudaErrorInvalidValue;
-    if (g.ag.on) {  // A gathered where it is stored: only the resident-B' kernel reads it so
-        if (!tc2_resident_b(g) || g.ag.run < 8 || g.ag.run > 11 || g.ag.nblk != 1 << (11 - g.ag.run))
+    if (g.ag.on) {  // A gathered where it is stored
+        if (g.ag.run < 6 || g.ag.run > 11 || g.ag.nblk != 1 << (11 - g.ag.run) || g.kb > 16 || g.a_div > 1)
             return cudaErrorInvalidValue;
-        return g.nb == 6 ? run_tc2kb<128, true>(g, st) : run_tc2kb<64, true>(g, st);
+        if (tc2_resident_b(g)) return g.nb == 6 ? run_tc2kb<128, true>(g, st) : run_tc2kb<64, true>(g, st);
+        return g.nb >= 6 ? run_tc2<128, true>(g, st) : run_tc2<64, true>(g, st);
     }
     // N = 32 complex per item: two items per 128-column tile when their B rows are contiguous and
     // they read the same A (shared, or per slice with an even number of items per slice)
     const int64_t NK = (1ll << g.nb) * (1ll << g.kb);
     const bool pack2 = g.nb == 5 && g.b_is == NK && g.b_div <= 1 && g.n_items % 2 == 0 &&
                        (g.a_is == 0 || (g.a_div > 1 && g.a_div % 2 == 0));
-    if (pack2) return run_tc2<128>(g, st, true);
+    if (pack2) return run_tc2<128, false>(g, st, true);
     if (tc2_resident_b(g)) return g.nb == 6 ? run_tc2kb<128, false>(g, st) : run_tc2kb<64, false>(g, st);
-    return g.nb >= 6 ? run_tc2<128>(g, st) : run_tc2<64>(g, st);
+    return g.nb >= 6 ? run_tc2<128, false>(g, st) : run_tc2<64, false>(g, st);
 }
 
 // B shared by every item, one tile wide (2N = BN), its B' small enough to stay resident, and A not
