@@ -228,11 +228,14 @@ int qx_submit_part(qx_handle h, const uint8_t* d_bitstrings, int64_t n_bits, int
                    int32_t first, int32_t last, double* d_amps_out, double* h_amps_out, int64_t* req_out);
 
 /* Graph replay (on by default): a call of qx_contract / qx_contract_device /
- * qx_contract_slices[_device] that repeats the previous call's device
- * buffers, bitstring count and slice range is captured once as a CUDA graph
- * and replayed afterwards (the contents of the buffers may change; the
- * pointers and sizes may not).  Not used on the legacy default stream or
- * while profiling.  enable = 0 turns it off and drops the captured graph. */
+ * qx_contract_slices[_device] that repeats the previous call's bitstring
+ * count and slice range is captured once as a CUDA graph and replayed
+ * afterwards, on the caller's buffers where they are the first call's, else
+ * on the workspace's own with a copy before and after (contents and buffers
+ * may change from call to call; the sizes may not).  The capture runs on a
+ * stream of the handle, so the legacy default stream replays too.  Not used
+ * while profiling or while the caller captures the handle's stream.
+ * enable = 0 turns it off and drops the captured graphs. */
 int qx_set_graphs(qx_handle h, int enable);
 
 /* Memoised invariant intermediates (the checkpoint reuse the paper's outlook
