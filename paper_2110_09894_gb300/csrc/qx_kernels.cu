@@ -1039,7 +1039,7 @@ static int skinny_smem(const SkinnyShape& sh) {
 }
 
 // the CTA shape of a skinny product, or false when it is not one
-static bool skinny_shape(int mb, int nb, int kb, SkinnyShape* sh) {
+static bool skinny_shape(int mb, int nb, int kb, int64_t n_items, SkinnyShape* sh) {
     sh->lb = std::max(mb, nb);
     sh->sb = std::min(mb, nb);
     sh->kb = kb;
@@ -1058,6 +1058,14 @@ static bool skinny_shape(int mb, int nb, int kb, SkinnyShape* sh) {
                 break;
             }
         }
+    // fewer CTAs than SMs: shorter pieces of the long side, with more chunks of K side by side (one
+    // product of 2 x 128 x 512: 26.3 us in one CTA, 6.2 in 32)
+    if ((n_items >> sh->items) << (sh->lb - sh->lr) < sm_count()) {
+        sh->items = 0;
+        while (sh->lr > 2 && n_items << (sh->lb - sh->lr) < sm_count()) --sh->lr;
+        sh->g = std::min(kb - sh->kw, 8 - sh->sb - sh->lr);
+        while (skinny_smem(*sh) > kSkinnySmem && sh->g) --sh->g;
+    }
     return skinny_smem(*sh) <= kSkinnySmem;
 }
 
@@ -1325,21 +1333,27 @@ cudaError_t launch_gemm_c64(const float2* a, int64_t a_is, bool a_kmajor, const 
         // the narrow tiles are CTAs of one or two warps: below 512 of them the 256-thread tiles of
         // k_gemm_c64 are faster (300 products of 32 x 32 x 128: 12.8 us against 22.6; 512 tiles of 32 x 64
         // x 128: 37.6 against 33.3)
-        if (mb > 5 && nb > 5) return QX_PACKED(64, 64);
+        if (mb > 5 && nb > 5 && n_items << (mb + nb - 12) >= sm_count()) return QX_PACKED(64, 64);
         if ((((1ll << mb) / (mb == 5 ? 32 : 64)) * ((1ll << nb) / (nb == 5 ? 32 : 64))) * n_items >= 512) {
             if (nb == 5) return mb == 5 ? QX_PACKED(32, 32) : QX_PACKED(64, 32);
             return QX_PACKED(32, 64);
         }
 #undef QX_PACKED
     }
-    const int bmb = mb >= 6 ? 6 : mb >= 5 ? 5 : 4;  // tile edge 64 / 32 / 16
-    const int bnb = nb >= 6 ? 6 : nb >= 5 ? 5 : 4;
-    const int64_t tm = ((1ll << mb) + (1 << bmb) - 1) >> bmb, tn = ((1ll << nb) + (1 << bnb) - 1) >> bnb;
+    int bmb = mb >= 6 ? 6 : mb >= 5 ? 5 : 4;  // tile edge 64 / 32 / 16
+    int bnb = nb >= 6 ? 6 : nb >= 5 ? 5 : 4;
+    auto tiles = [](int b, int tb) { return ((1ll << b) + (1 << tb) - 1) >> tb; };
     SkinnyShape sh;  // see k_gemm_skinny for where the line lies
-    if ((std::min(mb, nb) <= 2 || mb + nb <= 6 || (kb >= 8 && tm * tn * n_items < 2 * sm_count())) &&
-        skinny_shape(mb, nb, kb, &sh))
+    if ((std::min(mb, nb) <= 2 || mb + nb <= 6 ||
+         (kb >= 8 && tiles(mb, bmb) * tiles(nb, bnb) * n_items < 2 * sm_count())) &&
+        skinny_shape(mb, nb, kb, n_items, &sh))
         return gemm_skinny(sh, mb < nb, st, a, a_is, a_kmajor, b, b_is, b_kmajor, c, c_is, n_items, om, a_div, b_div);
-    dim3 grid((unsigned)(tm * tn), (unsigned)n_items);
+    // fewer tiles than SMs: smaller ones, on more SMs, each with less of the same serial sums.  One product:
+    // 128 x 512 x 128 20.6 -> 8.3 us, 64 x 64 x 64 12.3 -> 6.2, 64 x 64 x 4096 530 -> 131; 68 tiles of 64 x 64
+    // (17 products of 128 x 128 x 128) 20.6 -> 12.5.  Smaller ones again from 152 on lose: 19.0 there.
+    while (tiles(mb, bmb) * tiles(nb, bnb) * n_items < sm_count() && (bmb > 4 || bnb > 4)) --(bmb >= bnb ? bmb : bnb);
+    const int64_t tn = tiles(nb, bnb);
+    dim3 grid((unsigned)(tiles(mb, bmb) * tn), (unsigned)n_items);
 #define QX_GEMM_CASE(X, Y)                                                                            \
     if (bmb == X && bnb == Y) {                                                                       \
         gemm_tile<(1 << X), (1 << Y)>(grid, st, a, a_is, a_kmajor, b, b_is, b_kmajor, c, c_is, mb, nb, kb, \
