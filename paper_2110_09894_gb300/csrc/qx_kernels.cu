@@ -1142,7 +1142,10 @@ __global__ void __launch_bounds__(256) k_dot_c64(const float2* __restrict__ A, i
 // A step that contracts every leg with one operand stored in another leg order: per pair
 // C = sum_k A[k] B[p(k)], B read through the permutation's tiles (as k_permute: a tile in input
 // order into shared memory, then walked in A's order), so the permuted copy of B never goes to HBM.
-// One CTA per pair; per-thread FP32 partials, then a fixed-order tree.
+// One CTA per pair; per-thread FP32 partials, then a fixed-order tree.  Bound by HBM latency: a thread's 16
+// loads of an operand are issued together (B's, then A's into the same registers while B settles in
+// shared memory), four CTAs an SM.  16384 pairs of 8192 entries, 2.1 GB: 542 us with the loads one by
+// one, 549 with both operands in registers (two CTAs an SM), 428 so (5.0 TB/s).
 __global__ void __launch_bounds__(256, 4) k_dot_perm(const PermDesc d, const PermTables tb, const ItemCtx ic,
                                                   const float2* __restrict__ A, int64_t a_is, float2* __restrict__ C,
                                                   int64_t c_is, int a_div) {
@@ -1350,8 +1353,11 @@ cudaError_t launch_gemm_c64(const float2* a, int64_t a_is, bool a_kmajor, const 
         return gemm_skinny(sh, mb < nb, st, a, a_is, a_kmajor, b, b_is, b_kmajor, c, c_is, n_items, om, a_div, b_div);
     // fewer tiles than SMs: smaller ones, on more SMs, each with less of the same serial sums.  One product:
     // 128 x 512 x 128 20.6 -> 8.3 us, 64 x 64 x 64 12.3 -> 6.2, 64 x 64 x 4096 530 -> 131; 68 tiles of 64 x 64
-    // (17 products of 128 x 128 x 128) 20.6 -> 12.5.  Smaller ones again from 152 on lose: 19.0 there.
-    while (tiles(mb, bmb) * tiles(nb, bnb) * n_items < sm_count() && (bmb > 4 || bnb > 4)) --(bmb >= bnb ? bmb : bnb);
+    // (17 products of 128 x 128 x 128) 20.6 -> 12.5.  Smaller ones again from 152 on lose (19.0 there), and
+    // tiles of 32 do from 76 on: 120 products of 32 x 32 x 64 6.3 us, halved 8.2.
+    while (tiles(mb, bmb) * tiles(nb, bnb) * n_items < (std::max(bmb, bnb) == 6 ? sm_count() : sm_count() / 2) &&
+           (bmb > 4 || bnb > 4))
+        --(bmb >= bnb ? bmb : bnb);
     const int64_t tn = tiles(nb, bnb);
     dim3 grid((unsigned)(tiles(mb, bmb) * tn), (unsigned)n_items);
 #define QX_GEMM_CASE(X, Y)                                                                            \
