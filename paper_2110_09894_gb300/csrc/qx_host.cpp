@@ -987,28 +987,34 @@ static int compile_plan(qx_ctx* h, const int64_t* order, int64_t n_steps, const 
         // ones.  Measured, GEMM + permute before and GEMM alone after: one tile, m=14 k=6 n=6 per pair
         // 1225 + 1000 -> 1320 us (1024 items); two tiles, m=11 k=5 n=7 200 -> 152 us (300 items); four
         // tiles, m=8 k=12 n=8 3575 + 1030 -> 5250 us, so that one keeps its permute.
-        const int fa_n = (int)fA.size();
-        int a_gather = direct && fB.size() <= 7 && best.pa && GA.level == level && !GA.leaf && GA.fix.empty() &&
-                       fa_n + kb == (int)GA.legs.size() && fa_n <= kMaxRank && kb <= 16;
+        // (Apart from the resident-B' kernel's long blocks, the product's legs are ordered as for a permuted
+        // A: another order would change the order of later sums, and with it the amplitudes' last bits.)
+        const int fa_n = (int)fA.size(), fb_n = (int)fB.size();
+        const bool gatherable = direct && fb_n <= 7 && best.pa && GA.level == level && !GA.leaf && GA.fix.empty() &&
+                                fa_n + kb == (int)GA.legs.size() && fa_n <= kMaxRank && kb <= 16;
+        const bool resident = GB.level == 0 && ((fb_n == 6 && kb <= 6) || (fb_n == 5 && kb <= 7));
         std::vector<int8_t> ag_m, ag_k;
-        if (a_gather) {
+        auto gather_run = [&] {  // entries of a block, log2; 0 where A's tile can't be gathered
             auto pos_of = [&](int leg) {
                 return (int8_t)GA.pos[std::find(GA.legs.begin(), GA.legs.end(), leg) - GA.legs.begin()];
             };
+            ag_m.clear();
+            ag_k.clear();
             for (int i = 0; i < fa_n; ++i) ag_m.push_back(pos_of(fA[fa_n - 1 - i]));
             for (int i = 0; i < kb; ++i) ag_k.push_back(pos_of(best.S[kb - 1 - i]));
             AGather probe{};
             for (int i = 0; i < fa_n; ++i) probe.mpos[i] = ag_m[i];
             for (int i = 0; i < kb; ++i) probe.kpos[i] = ag_k[i];
-            const int fb_n = (int)fB.size();
-            const bool resident = GB.level == 0 && ((fb_n == 6 && kb <= 6) || (fb_n == 5 && kb <= 7));
-            a_gather = !agather_tile(&probe, fa_n, kb) ? 0 : resident && probe.run >= 8 ? 1 : 2;
-        }
-        if (a_gather) {
-            best.pa = false;
-            best.akm = true;
-        }
+            return agather_tile(&probe, fa_n, kb) ? probe.run : 0;
+        };
+        int a_gather = gatherable && resident && gather_run() >= 8 ? 1 : 0;
+        if (a_gather) best.pa = false;
         lay_out(t, fA, best.pa, fB, best.pb);
+        if (gatherable && !a_gather && gather_run() >= 6) {
+            a_gather = 2;
+            best.pa = false;
+        }
+        if (a_gather) best.akm = true;
         // the SIMT GEMM places its product with whole 128-byte runs along columns (16 complex); the
         // tensor-core kernels and the dot kernel store their natural layout (measured on GB300: placed
         // tensor-core stores and shorter SIMT runs cost more than the permutes they save)
@@ -2480,11 +2486,10 @@ static int contract_graph(qx_ctx* h, const uint8_t* d_bits, int64_t n_bits, int6
         gc.batches = h->last_batches;
     }
     if (!same && d_bits != w_bits)
-        CUDA_TRY(h, cudaMemcpyAsync(w_bits, d_bits, (size_t)(n_bits * h->nq), cudaMemcpyDeviceToDevice, h->stream));
+        CUDA_TRY(h, cudaMemcpyAsync(w_bits, d_bits, (size_t)(n_bits * h->nq), cudaMemcpyDefault, h->stream));
     CUDA_TRY(h, cudaGraphLaunch(*exec, h->stream));
     if (!same && d_amps != w_amps && h->part_final)
-        CUDA_TRY(h, cudaMemcpyAsync(d_amps, w_amps, (size_t)(n_bits << n_open(h)) * 16, cudaMemcpyDeviceToDevice,
-                                    h->stream));
+        CUDA_TRY(h, cudaMemcpyAsync(d_amps, w_amps, (size_t)(n_bits << n_open(h)) * 16, cudaMemcpyDefault, h->stream));
     h->last_flops = gc.flops;
     h->last_launches = gc.launches;
     h->last_batches = gc.batches;
