@@ -137,8 +137,11 @@ struct qx_ctx {
     int64_t n_slices = 1;
     double flops_inv = 0, flops_slice = 0, flops_item = 0;
 
+    int32_t plan_exec = 0;   // executor the plan was compiled for: decides its storage rules
+    int32_t bound_exec = 0;  // executor the bound workspace was laid out for (regions of the persistent kernel)
+
     // persistent executor program (variant ops, in order)
-    bool persist_ok = false;
+    bool persist_ok = false, persist_built = false;
     int64_t persist_entries = 0;  // scratch of one CTA: the tensors of a pair, per-slice ones among them
     std::vector<POp> pops;      // per-pair ops
     std::vector<POp> pops_inv;  // invariant ops (prologue program)
@@ -498,6 +501,7 @@ static int64_t assign_scratch(qx_ctx* h) {
 }
 
 static void build_persistent_program(qx_ctx* h);
+static bool persist_program(qx_ctx* h);
 static void choose_segments(qx_ctx* h);
 static void build_segments(qx_ctx* h);
 static void finish_layout(qx_ctx* h, bool segs);
@@ -560,6 +564,7 @@ static int compile_plan(qx_ctx* h, const int64_t* order, int64_t n_steps, const 
     if (n_sliced < 0 || n_sliced > 40) return fail(h, QX_EINVAL, "n_sliced %d out of range [0, 40]", n_sliced);
     // Intermediates that depend on the slice but on no output bit are computed once per slice and
     // shared by every bitstring of it (the persistent kernel runs them once per pair).
+    h->plan_exec = h->opt.executor;
     const bool slice_level = h->opt.executor != 2 && !h->opt.no_slice_level;
     std::vector<int> fixsrc(h->n_bonds, INT32_MIN);  // source of each fixed bond
     for (int j = 0; j < n_sliced; ++j) {
@@ -1159,15 +1164,12 @@ static int compile_plan(qx_ctx* h, const int64_t* order, int64_t n_steps, const 
 // whose operands from outside live until the segment's last step (and whose results in the prologue
 // live from the start); without them every step is a launch of its own, which needs the least memory.
 static void finish_layout(qx_ctx* h, bool segs) {
-    h->segs_on = segs && h->opt.executor != 2;
+    h->segs_on = segs && h->plan_exec != 2;
     h->stor = h->stor0;
     choose_segments(h);
     h->item_entries = std::max<int64_t>(assign_offsets(h, 2), kAlignEntries);
     h->slice_entries = assign_offsets(h, 1);
-    if (h->opt.executor >= 2) {
-        h->persist_entries = std::max<int64_t>(assign_scratch(h), kAlignEntries);
-    }
-    if (h->opt.executor < 2) {
+    if (h->plan_exec < 2) {
         // a small invariant region gets no reuse: then the only hazards between invariant steps are
         // their data dependencies
         int64_t tot = 0;
@@ -1182,7 +1184,8 @@ static void finish_layout(qx_ctx* h, bool segs) {
     }
     h->inv_entries = assign_offsets(h, 0);
     compute_deps(h);
-    build_persistent_program(h);
+    h->persist_ok = h->persist_built = false;
+    if (h->plan_exec >= 2 || h->opt.executor >= 2) persist_program(h);
     build_segments(h);
 }
 
@@ -1201,6 +1204,7 @@ static bool persist_active(const qx_ctx* h) {
 static bool persist_member(const qx_ctx* h) { return h->persist_ok && h->opt.executor >= 2; }
 
 static void layout(qx_ctx* h, int64_t max_bits, int64_t* fixed_bytes) {
+    if (h->opt.executor >= 2) persist_program(h);
     int64_t off = 0;
     h->off_err = off;  // device error flag (int)
     off += 256;
@@ -1262,16 +1266,18 @@ static bool fit_regions(const qx_ctx* h, int64_t avail, int64_t max_bits, int64_
 static bool fit_layout(qx_ctx* h, int64_t bytes, const int64_t* batch_bytes, int64_t max_bits, int64_t* fixed,
                        int64_t* items, int64_t* slices) {
     for (bool segs : {true, false}) {
-        if (h->opt.executor != 2 && h->segs_on != segs) finish_layout(h, segs);
+        if (h->plan_exec != 2 && h->segs_on != segs) finish_layout(h, segs);
         layout(h, max_bits, fixed);
-        if (h->opt.executor == 3) {  // a group member's own batch region is one pair's, its group's scratch serves runs
-            *items = *slices = 1;
+        if (h->opt.executor == 3) {
+            // a group member runs in its group's scratch.  Batch regions of its own are for a handle that is
+            // given another executor later: none (such a call is refused) where they don't fit
+            if (!fit_regions(h, bytes - *fixed, max_bits, items, slices)) *items = *slices = 0;
             if (bytes - *fixed >= h->persist_entries * 8) return true;
             continue;
         }
         const bool room = !batch_bytes || *fixed <= bytes;
         if (room && fit_regions(h, batch_bytes ? *batch_bytes : bytes - *fixed, max_bits, items, slices)) return true;
-        if (h->opt.executor == 2) return false;
+        if (h->plan_exec == 2) return false;
     }
     return false;
 }
@@ -1475,7 +1481,7 @@ static POp to_pop(const qx_ctx* h, const Op& op) {
 
 static void build_persistent_program(qx_ctx* h) {
     h->persist_ok = false;
-    if (h->opt.executor < 2) return;
+    h->persist_built = true;
     h->pops.clear();
     h->pops_inv.clear();
     for (const Op& op : h->ops)
@@ -1492,6 +1498,16 @@ static void build_persistent_program(qx_ctx* h) {
         h->pobit_leg[ob] = (int8_t)(std::find(R.legs.begin(), R.legs.end(), wire) - R.legs.begin());
     }
     h->persist_ok = true;
+}
+
+// Whether the plan has a persistent program; made when first asked for, as the executor may be chosen
+// after the plan was set.
+static bool persist_program(qx_ctx* h) {
+    if (!h->persist_built) {
+        h->persist_entries = std::max<int64_t>(assign_scratch(h), kAlignEntries);
+        build_persistent_program(h);
+    }
+    return h->persist_ok;
 }
 
 static double op_bytes(const qx_ctx* h, const Op& op, int64_t n_items, int64_t n_b = 1);
@@ -2320,9 +2336,15 @@ static int contract_impl(qx_ctx* h, const uint8_t* d_bits, int64_t n_bits, int64
     double* acc = (double*)(h->ws + h->off_acc);
     CUDA_TRY(h, cudaMemsetAsync(h->ws + h->off_err, 0, sizeof(int), h->stream));
     const int mode = in_group ? 1 : h->opt.executor;
+    if (mode >= 2) persist_program(h);
     if (mode >= 2 && !persist_active(h))
         return fail(h, QX_EINVAL, mode == 3 ? "a group member contracts only through qx_group_run"
                                             : "the persistent executor does not apply to this plan and precision form");
+    // the executor may have been changed since the workspace was laid out
+    if (mode == 2 && h->bound_exec != 2)
+        return fail(h, QX_ESTATE, "the workspace was bound for another executor; bind it again for the persistent one");
+    if (mode < 2 && h->items_cap < 1)
+        return fail(h, QX_ENOMEM, "the workspace was bound for a group member and holds no (slice, bitstring) pair");
     if (mode == 2) {
         if (!h->part_clear || !h->part_final)
             return fail(h, QX_EINVAL, "parts of a slice sum need the batched executor");
@@ -2617,12 +2639,9 @@ int qx_workspace_size(qx_handle h, int64_t max_bits, int64_t items, int64_t* byt
     if (items < 1) items = 1;
     int64_t fixed;
     layout(h, max_bits, &fixed);
-    if (h->opt.executor == 3) {
-        *bytes_out = fixed + items * h->persist_entries * 8;
-        return QX_OK;
-    }
     const int64_t slices = h->slice_entries ? std::min<int64_t>(h->n_slices, items) : 0;
     *bytes_out = fixed + align_up(slices * h->slice_entries * 8, 256) + items * h->item_entries * 8;
+    if (h->opt.executor == 3) *bytes_out = std::max(*bytes_out, fixed + items * h->persist_entries * 8);
     return QX_OK;
 }
 
@@ -2645,6 +2664,7 @@ int qx_bind_workspace(qx_handle h, void* dptr, int64_t bytes, int64_t max_bits) 
     h->ws = (char*)dptr;
     h->ws_bytes = bytes;
     h->max_bits = max_bits;
+    h->bound_exec = h->opt.executor;
     place_regions(h, fixed, items, slices);
     h->leaves_on_device = false;
     h->pops_on_device = false;
@@ -2688,6 +2708,7 @@ int qx_bind_workspace_parts(qx_handle h, void* d_fixed, int64_t fixed_bytes, voi
     h->wb = (char*)d_batch;
     h->ws_bytes = fixed_bytes;
     h->max_bits = max_bits;
+    h->bound_exec = h->opt.executor;
     place_regions(h, 0, items, slices);
     h->leaves_on_device = false;
     h->pops_on_device = false;
@@ -3056,10 +3077,11 @@ int qx_internal_contract_in(qx_ctx* h, char* buf, int64_t buf_bytes, const uint8
         bool leaves_on_device;
         int64_t off_pops, off_counter, off_results, off_pscratch, off_pops_inv, off_wave;
         bool pops_on_device, segs_on_device, inv_ready;
+        int32_t bound_exec;
     } const saved = {h->ws,        h->ws_bytes, h->ws_owned,    h->max_bits,    h->off_err,    h->off_leaf,
                      h->off_bits,  h->off_acc,  h->off_amps,    h->off_inv,     h->off_item,   h->items_cap,
                      h->off_slice, h->slices_cap, h->leaves_on_device, h->off_pops, h->off_counter, h->off_results, h->off_pscratch,
-                     h->off_pops_inv, h->off_wave, h->pops_on_device, h->segs_on_device, h->inv_ready};
+                     h->off_pops_inv, h->off_wave, h->pops_on_device, h->segs_on_device, h->inv_ready, h->bound_exec};
     int64_t fixed, items = 0, slices = 0;
     const bool saved_segs = h->segs_on;
     const bool fits = fit_layout(h, buf_bytes, nullptr, n_bits, &fixed, &items, &slices);
@@ -3089,6 +3111,7 @@ int qx_internal_contract_in(qx_ctx* h, char* buf, int64_t buf_bytes, const uint8
         h->off_wave = saved.off_wave;
         h->segs_on_device = saved.segs_on_device;
         h->inv_ready = saved.inv_ready;
+        h->bound_exec = saved.bound_exec;
     };
     if (!fits) {
         restore();
@@ -3102,6 +3125,7 @@ int qx_internal_contract_in(qx_ctx* h, char* buf, int64_t buf_bytes, const uint8
     h->ws_bytes = buf_bytes;
     h->ws_owned = false;
     h->max_bits = n_bits;
+    h->bound_exec = h->opt.executor;
     place_regions(h, fixed, items, slices);
     h->leaves_on_device = false;
     h->pops_on_device = false;
@@ -3269,7 +3293,7 @@ int qx_group_create(qx_group_t* out, qx_handle* hs, int32_t n, const uint8_t* co
         const char* why = nullptr;
         if (!h) why = "null handle";
         else if (!h->have_plan || !h->ws) why = "every handle needs a plan and a bound workspace";
-        else if (h->opt.executor != 3 || !h->persist_ok)
+        else if (h->opt.executor != 3 || h->bound_exec < 2 || !h->persist_ok)
             why = "every handle must be created with executor 3 and a plan without tensor-core steps";
         else if (h->device != hs[0]->device) why = "handles on different devices";
         else if (n_bits[i] < 1 || n_bits[i] > h->max_bits) why = "bitstring count outside the handle's workspace";
