@@ -100,9 +100,16 @@ struct Op {
 
 struct SegPlan;
 
+// Where the parts of the workspace lie (layout, place_regions)
+struct Offsets {
+    int64_t off_err = 0, off_leaf = 0, off_bits = 0, off_acc = 0, off_amps = 0, off_inv = 0, off_item = 0;
+    int64_t off_slice = 0, off_wave = 0;
+    int64_t off_pops = 0, off_counter = 0, off_results = 0, off_pscratch = 0, off_pops_inv = 0;
+};
+
 }  // namespace
 
-struct qx_ctx {
+struct qx_ctx : Offsets {
     int device = 0;
     cudaStream_t stream = nullptr;
     void* d_small = nullptr;  // 256 device bytes for small results (sampler counts), allocated on first use
@@ -184,10 +191,7 @@ struct qx_ctx {
     int64_t ws_bytes = 0;
     bool ws_owned = false;
     int64_t max_bits = 0;
-    int64_t off_err = 0, off_leaf = 0, off_bits = 0, off_acc = 0, off_amps = 0, off_inv = 0, off_item = 0;
-    int64_t off_slice = 0, slices_cap = 0;  // per-slice region: room for slices_cap slices
-    int64_t off_pops = 0, off_counter = 0, off_results = 0, off_pscratch = 0, off_pops_inv = 0, off_wave = 0;
-    int64_t items_cap = 0;
+    int64_t items_cap = 0, slices_cap = 0;  // pairs and slices that the batch regions have room for
     bool leaves_on_device = false;
 
     // stats
@@ -1236,6 +1240,15 @@ static void layout(qx_ctx* h, int64_t max_bits, int64_t* fixed_bytes) {
     off += align_up((int64_t)h->seg_blob.size(), 256);
     h->off_slice = h->off_item = off;
     *fixed_bytes = off;
+}
+
+// The fixed part's size alone: the handle's own workspace stays as it was laid out.
+static int64_t fixed_size(qx_ctx* h, int64_t max_bits) {
+    const Offsets bound = *h;
+    int64_t bytes;
+    layout(h, max_bits, &bytes);
+    static_cast<Offsets&>(*h) = bound;
+    return bytes;
 }
 
 // Split the bytes after the fixed part between the per-slice and the per-pair region: as many
@@ -2637,8 +2650,7 @@ int qx_workspace_size(qx_handle h, int64_t max_bits, int64_t items, int64_t* byt
     if (!h->have_plan) return fail(h, QX_ESTATE, "qx_workspace_size before qx_set_plan");
     if (max_bits < 1) return fail(h, QX_EINVAL, "max_bits < 1");
     if (items < 1) items = 1;
-    int64_t fixed;
-    layout(h, max_bits, &fixed);
+    const int64_t fixed = fixed_size(h, max_bits);
     const int64_t slices = h->slice_entries ? std::min<int64_t>(h->n_slices, items) : 0;
     *bytes_out = fixed + align_up(slices * h->slice_entries * 8, 256) + items * h->item_entries * 8;
     if (h->opt.executor == 3) *bytes_out = std::max(*bytes_out, fixed + items * h->persist_entries * 8);
@@ -2677,10 +2689,8 @@ int qx_workspace_parts(qx_handle h, int64_t max_bits, int64_t items, int64_t* fi
     if (!h->have_plan) return fail(h, QX_ESTATE, "qx_workspace_parts before qx_set_plan");
     if (max_bits < 1) return fail(h, QX_EINVAL, "max_bits < 1");
     if (items < 1) items = 1;
-    int64_t fixed;
-    layout(h, max_bits, &fixed);
+    *fixed_bytes = fixed_size(h, max_bits);
     const int64_t slices = h->slice_entries ? std::min<int64_t>(h->n_slices, items) : 0;
-    *fixed_bytes = fixed;
     *batch_bytes = align_up(slices * h->slice_entries * 8, 256) + items * h->item_entries * 8;
     return QX_OK;
 }
