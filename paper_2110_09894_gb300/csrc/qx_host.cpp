@@ -3030,7 +3030,8 @@ int qx_device_status(qx_handle h) {
     CUDA_TRY(h, cudaStreamSynchronize(h->stream));
     h->static_err = nullptr;
     if (flag) {
-        h->inv_ready = false;  // the kept intermediates may be incomplete
+        h->inv_ready = false;  // the kept intermediates may be incomplete,
+        drop_graph(h);         // and a graph captured while they were kept doesn't compute them
         return fail(h, flag, "a bounded device wait expired; the result is invalid");
     }
     if (sflag) return fail(h, sflag, "a bounded device wait expired in a static-scratch call; the result is invalid");
