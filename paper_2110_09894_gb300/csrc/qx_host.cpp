@@ -2441,7 +2441,11 @@ static int contract_impl(qx_ctx* h, const uint8_t* d_bits, int64_t n_bits, int64
         if (e != cudaSuccess) return fail(h, QX_ECUDA, "finalize launch failed: %s", cudaGetErrorString(e));
         h->last_launches++;
     }
-    if (h->memo) h->inv_ready = true;
+    if (h->memo && !h->inv_ready) {  // kept once they are computed: a call that is only being captured hasn't run
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (h->stream && h->stream != cudaStreamLegacy) CUDA_TRY(h, cudaStreamIsCapturing(h->stream, &cap));
+        h->inv_ready = cap == cudaStreamCaptureStatusNone;
+    }
     return QX_OK;
 }
 

@@ -50,3 +50,31 @@ def test_a_reported_expiry_drops_graphs_without_the_invariant_steps(qx, fresh):
     assert call() == whole
     torch.cuda.synchronize()
     c.close()
+
+
+def test_a_captured_call_that_has_not_run_keeps_nothing(qx):
+    torch, c, d_bits, out = _contractor(qx, 8)
+    with torch.cuda.stream(c.stream):
+        want = c.contract_device(d_bits, out).clone()
+    whole = c.stats()["launches"]
+    torch.cuda.synchronize()
+    qx.qx_set_memo(c.h, True)
+    captured = torch.zeros_like(out)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=c.stream):
+        c.contract_device(d_bits, captured)
+    counts = []
+    for _ in range(2):
+        out.zero_()
+        torch.cuda.synchronize()
+        c.contract_device(d_bits, out)
+        counts.append(c.stats()["launches"])
+        torch.cuda.synchronize()
+        assert torch.equal(out, want)
+    assert counts[0] == whole > counts[1]
+    with torch.cuda.stream(c.stream):
+        graph.replay()  # holds the invariant steps itself
+    torch.cuda.synchronize()
+    assert torch.equal(captured, want)
+    qx.qx_device_status(c.h)
+    c.close()
