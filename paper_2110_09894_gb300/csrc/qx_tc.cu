@@ -255,6 +255,13 @@ __device__ __forceinline__ void mbar_wait_issued(uint64_t* b, uint32_t parity) {
     while (!mbar_try(b, parity))
         if (clock64() - t0 > kIssuedWaitCycles) return;
 }
+// Whether an earlier CTA of this contraction gave up: then the whole CTA leaves at its start.  One read
+// decides for all its threads.  The flag may be set between the reads of two warps; warps that stayed
+// while the one that sets up the mbarriers or TMEM had left would wait on whatever the SM's last CTA left
+// there, and free TMEM under MMAs in flight or address TMEM that nobody allocated.
+__device__ __forceinline__ bool gave_up(const int* err) {
+    return __syncthreads_or(threadIdx.x == 0 && *(volatile const int*)err);
+}
 // progress of another warp of the CTA: waits (bounded as mbar_wait) until *p has reached `stage`; stage
 // numbers compare modulo 2^32
 __device__ __forceinline__ void prog_set(int* p, int stage) {
@@ -474,7 +481,7 @@ __global__ void __launch_bounds__(TcTile<FORM, BN, ROWB>::THREADS, 1)
     __shared__ uint64_t full[STAGES], empty[STAGES], tfull[NTB], tempty[NTB], drain;
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
-    if (*(volatile const int*)err) return;  // an earlier CTA of this contraction gave up
+    if (gave_up(err)) return;
     uint8_t* base = (uint8_t*)(((uintptr_t)dyn + 1023) & ~(uintptr_t)1023);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nk = (K2 + BK - 1) / BK, np = (nk + SPD - 1) / SPD;
@@ -811,7 +818,7 @@ __global__ void __launch_bounds__(TC2_THREADS2, 1)
     __shared__ int abort_flag;
     __shared__ int16_t s_lrow[GA ? 128 : 1], s_lk[GA ? 16 : 1];  // GA: the slot offsets of rows / K entries
     __shared__ int conv_seen[2][4];  // per converter group and warp: the last stage whose slots it saw ready
-    if (*(volatile const int*)err) return;
+    if (gave_up(err)) return;
     uint8_t* base = (uint8_t*)(((uintptr_t)dyn + 1023) & ~(uintptr_t)1023);
     auto land = [&](int l) { return base + l * L::LAND; };
     auto mslot = [&](int m) { return base + NL * L::LAND + m * L::MSLOT; };
@@ -1237,7 +1244,7 @@ __global__ void __launch_bounds__(TC2_THREADS2, 1)
     __shared__ int abort_flag;
     __shared__ int conv_seen[2][4];  // per converter group and warp: the last A stage whose slots it saw ready
     __shared__ int16_t s_lrow[GA ? 128 : 1], s_lk[GA ? 16 : 1];  // GA: the slot offsets of rows / K entries
-    if (*(volatile const int*)err) return;
+    if (gave_up(err)) return;
     uint8_t* base = (uint8_t*)(((uintptr_t)dyn + 1023) & ~(uintptr_t)1023);
     auto land = [&](int l) { return base + l * L::LAND; };
     auto bslot = [&](int it) { return base + NL * L::LAND + it * L::BSLOT; };
