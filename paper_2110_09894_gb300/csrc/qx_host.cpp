@@ -182,7 +182,7 @@ struct qx_ctx : Offsets {
     std::vector<std::pair<int64_t, int64_t>> pair_life;  // their lifetimes when a CTA runs one pair's steps in order
     bool wave_ok = false;               // there is a prologue launch
     std::vector<int> chain_of_op;       // per op: its prologue segment, -1 if none
-    double wave_flops = 0, wave_bytes = 0;
+    double wave_flops = 0;
     bool segs_on_device = false;
     cudaEvent_t wave_ev = nullptr;
 
@@ -1732,7 +1732,7 @@ static void build_segments(qx_ctx* h) {
     h->seg_blob.clear();
     h->n_waves = 0;
     h->wave_ok = false;
-    h->wave_flops = h->wave_bytes = 0;
+    h->wave_flops = 0;
     h->chain_of_op.assign(h->ops.size(), -1);
     std::vector<int32_t> wave_offs;
     for (auto& sg : h->segs) {
@@ -1876,7 +1876,6 @@ static void build_segments(qx_ctx* h) {
             for (int i : sg.ops) h->chain_of_op[i] = h->n_waves;
             wave_offs.push_back((int32_t)sg.prog_off);
             h->wave_flops += sg.flops;
-            h->wave_bytes += sg.bytes;
             h->n_waves++;
         }
     }
@@ -1921,6 +1920,19 @@ static double op_bytes(const qx_ctx* h, const Op& op, int64_t n_items, int64_t n
     if (op.type == OP_SMALL) return c + node_b(op.x) + node_b(op.y);
     if (op.dot_perm) return c + stor_b(op.sa) + node_b(op.perm_src);
     return c + stor_b(op.sa) + stor_b(op.sb);
+}
+
+// Bytes that a segment's launch moves: the operands from outside it and the result (the steps' other
+// tensors stay in shared memory; op_bytes counts those of launches per step)
+static double seg_traffic(const qx_ctx* h, const qx_ctx::Seg& sg, int64_t n_items, int64_t n_b = 1) {
+    double bytes = 8.0 * (double)h->stor[h->ops[sg.ops.back()].dst].entries * (double)n_items;
+    for (const auto& t : sg.plan->in) {
+        const Op& op = h->ops[sg.ops[t.op]];
+        const int sid = seg_storage(h, op, t.side);
+        const int level = sid >= 0 ? h->stor[sid].level : h->nodes[op.type == OP_PERM ? op.src : t.side ? op.y : op.x].level;
+        bytes += 8.0 * (double)((int64_t)1 << t.bits) * copies(op, level, n_items, n_b);
+    }
+    return bytes;
 }
 
 static int run_op(qx_ctx* h, const Op& op, const ItemCtx& ic, int64_t n_items, cudaStream_t st) {
@@ -2215,13 +2227,15 @@ struct Dag {
         SegCtx c = seg_ctx(ic, 1, 0);
         c.prog = (const uint8_t*)(h->ws + h->off_wave);
         c.prog_off = (const int32_t*)(c.prog + h->wave_list);
+        double bytes = 0;
         for (const auto& sg : h->segs)
             if (sg.wave) {
+                bytes += seg_traffic(h, sg, 1);
                 c.prog_bytes = std::max(c.prog_bytes, sg.prog_bytes);
                 c.arena = std::max(c.arena, sg.arena);
             }
         size_t slot;
-        cudaError_t e = prof_begin(h, QX_KERNEL_WAVE, h->wave_flops, h->wave_bytes, &slot);
+        cudaError_t e = prof_begin(h, QX_KERNEL_WAVE, h->wave_flops, bytes, &slot);
         if (e == cudaSuccess) e = launch_seg(c, h->n_waves, 512, h->stream);
         if (e == cudaSuccess) e = prof_end(h, slot);
         if (e == cudaSuccess && on) e = cudaEventRecord(h->wave_ev, h->stream);
@@ -2238,7 +2252,8 @@ struct Dag {
         c.prog_bytes = sg.prog_bytes;
         c.arena = sg.arena;
         size_t slot;
-        cudaError_t e = prof_begin(h, QX_KERNEL_WAVE, sg.flops * (double)n_items, 0.0, &slot);
+        cudaError_t e = prof_begin(h, QX_KERNEL_WAVE, sg.flops * (double)n_items,
+                                   seg_traffic(h, sg, n_items, sg.level == 2 ? ic.n_b : 1), &slot);
         if (e == cudaSuccess) e = launch_seg(c, 1, seg_threads(n_items), st);
         if (e == cudaSuccess) e = prof_end(h, slot);
         if (e != cudaSuccess) return fail(h, QX_ECUDA, "segment launch failed: %s", cudaGetErrorString(e));
