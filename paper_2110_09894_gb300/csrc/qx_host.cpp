@@ -2977,6 +2977,12 @@ int qx_describe_plan(qx_handle h, char* buf, int64_t len, int64_t* needed) {
             snprintf(line, sizeof line, " seg=%d", h->seg_of[i]);
             out += line;
         }
+        if (h->seg_of[i] >= 0 && h->segs[h->seg_of[i]].ops.back() == (int)i) {
+            // what seg_pays weighs: stages, issue clocks per item, bytes per item of launches per step
+            const qx_ctx::Seg& sg = h->segs[h->seg_of[i]];
+            snprintf(line, sizeof line, " stages=%d clocks=%.0f step_bytes=%.0f", sg.n_stages, sg.warp_clocks, sg.bytes);
+            out += line;
+        }
         out += "\n";
     }
     if (needed) *needed = (int64_t)out.size() + 1;

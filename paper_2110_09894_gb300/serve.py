@@ -43,7 +43,7 @@ from dataclasses import dataclass, field
 import numpy as np
 
 from . import qx
-from .cost import launch_list_time
+from .cost import launch_list_time, launches
 
 
 @dataclass
@@ -161,8 +161,8 @@ class Server:
             sc.lane_bytes = qx.qx_workspace_size(h, max_bits, items)
             sc.servable = sc.lane_bytes <= self.budget
             desc = qx.qx_describe_plan(h)
-            lv = [ln.split()[3] for ln in desc.splitlines()]
-            sc.slice_ops, sc.pair_ops = lv.count("slice"), lv.count("pair")
+            lv = [level for level, _ in launches(desc, (1, min(sc.n_slices, items), items))]
+            sc.slice_ops, sc.pair_ops = lv.count(1), lv.count(2)
             t1 = launch_list_time(desc, sc.n_slices, 1)
             sc.est_b = max((launch_list_time(desc, sc.n_slices, 256) - t1) / 255.0, 0.0)
             sc.est_a = t1 - sc.est_b
