@@ -25,6 +25,11 @@ __device__ __forceinline__ void neumaier(double& s, double& c, double x) {
     c += (big - t) + small;
     s = t;
 }
+// An amplitude from its slice sum (re, im) and the circuit's scale factor (sr, si): component c (0: re, 1: im).
+// The roundings are written out, so that every kernel that ends a sum gives the same bits.
+__device__ __forceinline__ double scaled(int c, double re, double im, double sr, double si) {
+    return c == 0 ? __fma_rn(re, sr, -__dmul_rn(im, si)) : __fma_rn(re, si, __dmul_rn(im, sr));
+}
 #endif
 
 // The (slice, bitstring) pairs of one batch: item = s_local * n_b + b_local.

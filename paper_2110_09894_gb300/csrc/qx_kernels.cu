@@ -1440,8 +1440,8 @@ __global__ void k_finalize(const double* __restrict__ acc, double* __restrict__ 
     if (i >= n) return;
     const double re = acc[4 * i] + acc[4 * i + 2];
     const double im = acc[4 * i + 1] + acc[4 * i + 3];
-    amps[2 * i] = re * sr - im * si;
-    amps[2 * i + 1] = re * si + im * sr;
+    amps[2 * i] = scaled(0, re, im, sr, si);
+    amps[2 * i + 1] = scaled(1, re, im, sr, si);
 }
 
 cudaError_t launch_finalize(const double* acc, double* amps, int64_t n, double sr, double si, cudaStream_t st) {

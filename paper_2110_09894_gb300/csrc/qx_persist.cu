@@ -352,8 +352,7 @@ __device__ __forceinline__ void gsum_one(const GSum& g, int64_t local2, bool liv
     }
     const double mine = s + comp, other = __shfl_xor_sync(0xffffffffu, mine, 1);
     if (!live) return;
-    if (c == 0) g.amps[2 * local] = mine * g.sr - other * g.si;
-    else g.amps[2 * local + 1] = other * g.si + mine * g.sr;
+    g.amps[local2] = c == 0 ? scaled(0, mine, other, g.sr, g.si) : scaled(1, other, mine, g.sr, g.si);
 }
 
 __global__ void __launch_bounds__(kSumThreads) k_group_sum(const GSum* __restrict__ sums, int32_t n, int64_t total) {
