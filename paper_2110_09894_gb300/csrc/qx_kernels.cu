@@ -1039,7 +1039,7 @@ static int skinny_smem(const SkinnyShape& sh) {
 }
 
 // the CTA shape of a skinny product, or false when it is not one
-static bool skinny_shape(int mb, int nb, int kb, int64_t n_items, SkinnyShape* sh) {
+static bool skinny_shape(int mb, int nb, int kb, int64_t n_items, int sms, SkinnyShape* sh) {
     sh->lb = std::max(mb, nb);
     sh->sb = std::min(mb, nb);
     sh->kb = kb;
@@ -1060,9 +1060,9 @@ static bool skinny_shape(int mb, int nb, int kb, int64_t n_items, SkinnyShape* s
         }
     // fewer CTAs than SMs: shorter pieces of the long side, with more chunks of K side by side (one
     // product of 2 x 128 x 512: 26.3 us in one CTA, 6.2 in 32)
-    if ((n_items >> sh->items) << (sh->lb - sh->lr) < sm_count()) {
+    if ((n_items >> sh->items) << (sh->lb - sh->lr) < sms) {
         sh->items = 0;
-        while (sh->lr > 2 && n_items << (sh->lb - sh->lr) < sm_count()) --sh->lr;
+        while (sh->lr > 2 && n_items << (sh->lb - sh->lr) < sms) --sh->lr;
         sh->g = std::min(kb - sh->kw, 8 - sh->sb - sh->lr);
         while (skinny_smem(*sh) > kSkinnySmem && sh->g) --sh->g;
     }
@@ -1274,21 +1274,49 @@ static void gemm_tile(dim3 grid, cudaStream_t st, const float2* a, int64_t a_is,
                       int64_t b_is, bool bkm, float2* c, int64_t c_is, int mb, int nb, int kb, int tn,
                       const OutMap& om, int a_div, int b_div) {
     constexpr int smem = 2 * GBK * (BM + 1 + BN + 1) * (int)sizeof(float2);
-    if (smem > 48 * 1024) {
-        // opt in to more than 48 KB of dynamic shared memory, once per device
-        static uint64_t done[4] = {0, 0, 0, 0};
-        static std::mutex mu;
-        int dev = 0;
-        if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 256) {
-            std::lock_guard<std::mutex> lk(mu);
-            if (!((done[dev >> 6] >> (dev & 63)) & 1) &&
-                cudaFuncSetAttribute(k_gemm_c64<BM, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) ==
-                    cudaSuccess)
-                done[dev >> 6] |= 1ull << (dev & 63);
-        }
-    }
+    static_assert(smem <= 48 * 1024, "the default limit of dynamic shared memory");
     k_gemm_c64<BM, BN><<<grid, 256, smem, st>>>(a, a_is, akm, b, b_is, bkm, c, c_is, mb, nb, kb, tn, om, a_div,
                                                 b_div);
+}
+
+// The kernel that a complex64 product of 2^mb x 2^kb x 2^nb over n_items items takes on a GPU of `sms` SMs,
+// with its tile edges (log2).
+enum { GEMM_SMALL_K, GEMM_DOT, GEMM_PACKED, GEMM_SKINNY, GEMM_TILE };
+struct GemmRoute {
+    int kind, bm, bn;
+    SkinnyShape sh;
+};
+static GemmRoute gemm_route(int mb, int nb, int kb, int64_t n_items, int sms) {
+    GemmRoute r{};
+    auto is = [&](int kind, int bm, int bn) {
+        r.kind = kind;
+        r.bm = bm;
+        r.bn = bn;
+        return r;
+    };
+    auto tiles = [&](int bm, int bn) {
+        return (((1ll << mb) + (1 << bm) - 1) >> bm) * (((1ll << nb) + (1 << bn) - 1) >> bn) * n_items;
+    };
+    if (kb <= 2 && nb >= 5) return is(GEMM_SMALL_K, 0, 0);
+    if (mb + nb <= 4 && kb >= 8) return is(GEMM_DOT, mb, nb);
+    auto edge = [](int b) { return std::min(std::max(b, 4), 6); };  // 16, 32 or 64
+    int bm = edge(mb), bn = edge(nb);
+    // 64 x 64 tiles run on k_gemm_packed from one per SM on and are cut below (k_gemm_c64 has none): one
+    // line for both.  The narrow tiles are CTAs of one or two warps: below 512 of them the 256-thread
+    // tiles of k_gemm_c64 are faster (300 products of 32 x 32 x 128: 12.8 us against 22.6; 512 tiles of
+    // 32 x 64 x 128: 37.6 against 33.3)
+    const int whole = std::min(sms, 512);
+    if (mb >= 5 && nb >= 5 && tiles(bm, bn) >= (bm == 6 && bn == 6 ? whole : 512)) return is(GEMM_PACKED, bm, bn);
+    // see k_gemm_skinny for where the line lies
+    if ((std::min(mb, nb) <= 2 || mb + nb <= 6 || (kb >= 8 && tiles(bm, bn) < 2 * sms)) &&
+        skinny_shape(mb, nb, kb, n_items, sms, &r.sh))
+        return is(GEMM_SKINNY, 0, 0);
+    // fewer tiles than SMs: smaller ones, on more SMs, each with less of the same serial sums.  One product:
+    // 128 x 512 x 128 20.6 -> 8.3 us, 64 x 64 x 64 12.3 -> 6.2, 64 x 64 x 4096 530 -> 131; 68 tiles of 64 x 64
+    // (17 products of 128 x 128 x 128) 20.6 -> 12.5.  Smaller ones again from 152 on lose (19.0 there), and
+    // tiles of 32 do from 76 on: 120 products of 32 x 32 x 64 6.3 us, halved 8.2.
+    while (tiles(bm, bn) < (std::max(bm, bn) == 6 ? whole : sms / 2) && (bm > 4 || bn > 4)) --(bm >= bn ? bm : bn);
+    return is(GEMM_TILE, bm, bn);
 }
 
 cudaError_t launch_gemm_c64(const float2* a, int64_t a_is, bool a_kmajor, const float2* b, int64_t b_is,
@@ -1298,7 +1326,8 @@ cudaError_t launch_gemm_c64(const float2* a, int64_t a_is, bool a_kmajor, const 
     if (a_div < 1 || b_div < 1) return cudaErrorInvalidValue;
     OutMap om{};
     if (omp) om = *omp;
-    if (kb <= 2 && nb >= 5) {
+    const GemmRoute r = gemm_route(mb, nb, kb, n_items, sm_count());
+    if (r.kind == GEMM_SMALL_K) {
         // about 4096 outputs per CTA
         const int64_t M = (int64_t)1 << mb, N = (int64_t)1 << nb;
         const int64_t width = N < 256 ? N : 256;
@@ -1312,7 +1341,7 @@ cudaError_t launch_gemm_c64(const float2* a, int64_t a_is, bool a_kmajor, const 
         }
         return cudaGetLastError();
     }
-    if (mb + nb <= 4 && kb >= 8) {
+    if (r.kind == GEMM_DOT) {
         if (om.on) return cudaErrorInvalidValue;  // the dot kernel writes the natural layout only
         dim3 grid((unsigned)n_items);
 #define QX_DOT_CASE(X, Y)                                                                                   \
@@ -1327,41 +1356,24 @@ cudaError_t launch_gemm_c64(const float2* a, int64_t a_is, bool a_kmajor, const 
 #undef QX_DOT_CASE
         return cudaErrorInvalidValue;
     }
-    if (mb >= 5 && nb >= 5 && kb >= 3) {
-#define QX_PACKED(X, Y)                                                                                             \
-    (kb > 6 ? gemm_packed<X, Y, true>(st, a, a_is, a_kmajor, b, b_is, b_kmajor, c, c_is, mb, nb, kb, n_items, om,  \
-                                      a_div, b_div)                                                                \
-            : gemm_packed<X, Y, false>(st, a, a_is, a_kmajor, b, b_is, b_kmajor, c, c_is, mb, nb, kb, n_items, om, \
-                                       a_div, b_div))
-        // the narrow tiles are CTAs of one or two warps: below 512 of them the 256-thread tiles of
-        // k_gemm_c64 are faster (300 products of 32 x 32 x 128: 12.8 us against 22.6; 512 tiles of 32 x 64
-        // x 128: 37.6 against 33.3)
-        if (mb > 5 && nb > 5 && n_items << (mb + nb - 12) >= sm_count()) return QX_PACKED(64, 64);
-        if ((((1ll << mb) / (mb == 5 ? 32 : 64)) * ((1ll << nb) / (nb == 5 ? 32 : 64))) * n_items >= 512) {
-            if (nb == 5) return mb == 5 ? QX_PACKED(32, 32) : QX_PACKED(64, 32);
-            return QX_PACKED(32, 64);
-        }
-#undef QX_PACKED
+    if (r.kind == GEMM_PACKED) {
+#define QX_PACKED_CASE(X, Y)                                                                                        \
+    if (r.bm == X && r.bn == Y)                                                                                     \
+        return kb > 6 ? gemm_packed<1 << X, 1 << Y, true>(st, a, a_is, a_kmajor, b, b_is, b_kmajor, c, c_is, mb,    \
+                                                          nb, kb, n_items, om, a_div, b_div)                        \
+                      : gemm_packed<1 << X, 1 << Y, false>(st, a, a_is, a_kmajor, b, b_is, b_kmajor, c, c_is, mb,   \
+                                                           nb, kb, n_items, om, a_div, b_div);
+        QX_PACKED_CASE(6, 6) QX_PACKED_CASE(6, 5)
+        QX_PACKED_CASE(5, 6) QX_PACKED_CASE(5, 5)
+#undef QX_PACKED_CASE
+        return cudaErrorInvalidValue;
     }
-    int bmb = mb >= 6 ? 6 : mb >= 5 ? 5 : 4;  // tile edge 64 / 32 / 16
-    int bnb = nb >= 6 ? 6 : nb >= 5 ? 5 : 4;
-    auto tiles = [](int b, int tb) { return ((1ll << b) + (1 << tb) - 1) >> tb; };
-    SkinnyShape sh;  // see k_gemm_skinny for where the line lies
-    if ((std::min(mb, nb) <= 2 || mb + nb <= 6 ||
-         (kb >= 8 && tiles(mb, bmb) * tiles(nb, bnb) * n_items < 2 * sm_count())) &&
-        skinny_shape(mb, nb, kb, n_items, &sh))
-        return gemm_skinny(sh, mb < nb, st, a, a_is, a_kmajor, b, b_is, b_kmajor, c, c_is, n_items, om, a_div, b_div);
-    // fewer tiles than SMs: smaller ones, on more SMs, each with less of the same serial sums.  One product:
-    // 128 x 512 x 128 20.6 -> 8.3 us, 64 x 64 x 64 12.3 -> 6.2, 64 x 64 x 4096 530 -> 131; 68 tiles of 64 x 64
-    // (17 products of 128 x 128 x 128) 20.6 -> 12.5.  Smaller ones again from 152 on lose (19.0 there), and
-    // tiles of 32 do from 76 on: 120 products of 32 x 32 x 64 6.3 us, halved 8.2.
-    while (tiles(mb, bmb) * tiles(nb, bnb) * n_items < (std::max(bmb, bnb) == 6 ? sm_count() : sm_count() / 2) &&
-           (bmb > 4 || bnb > 4))
-        --(bmb >= bnb ? bmb : bnb);
-    const int64_t tn = tiles(nb, bnb);
-    dim3 grid((unsigned)(tiles(mb, bmb) * tn), (unsigned)n_items);
+    if (r.kind == GEMM_SKINNY)
+        return gemm_skinny(r.sh, mb < nb, st, a, a_is, a_kmajor, b, b_is, b_kmajor, c, c_is, n_items, om, a_div, b_div);
+    const int64_t tm = ((1ll << mb) + (1 << r.bm) - 1) >> r.bm, tn = ((1ll << nb) + (1 << r.bn) - 1) >> r.bn;
+    dim3 grid((unsigned)(tm * tn), (unsigned)n_items);
 #define QX_GEMM_CASE(X, Y)                                                                            \
-    if (bmb == X && bnb == Y) {                                                                       \
+    if (r.bm == X && r.bn == Y) {                                                                       \
         gemm_tile<(1 << X), (1 << Y)>(grid, st, a, a_is, a_kmajor, b, b_is, b_kmajor, c, c_is, mb, nb, kb, \
                                       (int)tn, om, a_div, b_div);                                     \
         return cudaGetLastError();                                                                    \
@@ -1371,6 +1383,12 @@ cudaError_t launch_gemm_c64(const float2* a, int64_t a_is, bool a_kmajor, const 
     QX_GEMM_CASE(4, 6) QX_GEMM_CASE(4, 5) QX_GEMM_CASE(4, 4)
 #undef QX_GEMM_CASE
     return cudaErrorInvalidValue;
+}
+
+// For the tests: 100 kind + 10 row edge + column edge of the kernel a product takes (gemm_route)
+extern "C" int qx_internal_gemm_route(int mb, int nb, int kb, int64_t n_items, int sms) {
+    const GemmRoute r = gemm_route(mb, nb, kb, n_items, sms);
+    return 100 * r.kind + 10 * r.bm + r.bn;
 }
 
 // ---------------------------------------------------------------------------------------------
