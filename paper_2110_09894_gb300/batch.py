@@ -3,9 +3,10 @@
 The slices and bitstrings of many circuits are independent units of work
 (Sec. IV-A's slice and bitstring levels of parallelism, across circuits).
 Members whose intermediates fit one CTA's scratch (at most 2^18 entries per
-(slice, bitstring) pair, no tensor-core step) run in the persistent group
-launch of the C ABI (qx_group_*: whole contractions per CTA, one FP64 sum);
-the others -- large intermediates, tensor-core products -- run on the batched
+(slice, bitstring) pair, no tensor-core step) form a group of the C ABI
+(qx_group_*): those with little work per pair run in its persistent launch
+(whole contractions per CTA, one FP64 sum), the group runs the others as
+launches over batches of pairs in its scratch; the heavy members -- large intermediates, tensor-core products -- run on the batched
 executor (one launch per step over many pairs, steps at their dependence
 level).  Everything is enqueued on one stream and captured as one CUDA graph,
 so a step of the whole workload is one graph launch.
@@ -22,7 +23,8 @@ LIGHT_MAX_PEAK = 18  # per-pair entries a persistent CTA's scratch holds (2^18 c
 class UnevenBatch:
     """workloads: objects with n_qubits, gates, open_mask, order, sliced, bitstrings, peak_rank.
 
-    precision applies to the heavy members (the persistent launch runs complex64);
+    precision applies to the heavy members (the group's members run in complex64, in its persistent
+    launch or as launches);
     settings maps a heavy member's index to autotuned Contractor options
     ({"max_items": .., "gemm_min_bits": ..}); mem_budget caps the heavy members'
     workspaces together (bytes, default 60% of the free device memory): each

@@ -1891,8 +1891,11 @@ static int seg_threads(int64_t n_items) { return n_items >= 2048 ? 128 : n_items
 // Whether running the segment beats a launch per step over n_items items.  A few items: the segment's
 // latency (a launch, its operands, 0.35 us a stage: 10 to 25 us measured) against the launches' (2.5 us
 // each, measured 3 to 5 and partly side by side).  Many items: the segment's issue time, 3.5 times its
-// estimated clocks (measured 189 and 420 us where 58 and 117 were estimated, on 16384 pairs: bank
-// conflicts of the strided reads), against the launches' bytes through HBM (62 and 133 us there).
+// estimated clocks (bank conflicts of the strided reads), against the launches' bytes through HBM.  The
+// 22 per-pair and per-slice segments of five plans, run as segments whatever the rule says: from 8192 to
+// 60000 items every further item costs 2.7 to 4.1 times its clocks, at 16384 items the whole 2.8 to 4.5
+// (checkpoint plan 659 us for 176, 12-qubit plan 595 for 215), at 2048 items 3.7 to 7.2, the latency
+// among them.  The rule is also asked on host-only handles, so it counts the SMs of a whole GB300.
 static bool seg_pays(const qx_ctx::Seg& sg, int64_t n_items) {
     const double lat = 4.0 + 0.35 * sg.n_stages;
     const double issue = 3.5 * (double)n_items * sg.warp_clocks / (152 * 4) / 1.9e3;
@@ -3207,7 +3210,9 @@ struct qx_group {
 
 // Estimated microseconds of a member on the persistent launch (its share of the GPU) and as launches.
 // The persistent kernel runs one pair per CTA, per-slice steps included, at about 12 TFLOP/s over the
-// GPU; launches cost 2.5 us each per batch, their flops at 35 TFLOP/s or their bytes at 4.5 TB/s.
+// GPU (measured 10.4 to 16.5 on members of 2176 to 14848 pairs; members of fewer pairs leave CTAs idle and
+// share the launch with others); launches cost 2.5 us each per batch, their flops at 35 TFLOP/s (measured
+// 33 to 40 on members of large products) or their bytes at 4.5 TB/s.
 static double persist_us(const qx_ctx* h, int64_t n_bits) {
     return (double)(h->n_slices * n_bits) * (h->flops_slice + h->flops_item) / 12e6;
 }

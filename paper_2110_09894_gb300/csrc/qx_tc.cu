@@ -1633,6 +1633,7 @@ static cudaError_t run_prep(const TcArgs& g, cudaStream_t st) {
         cudaError_t e = cudaMemsetAsync(g.amax, 0, 2 * sizeof(float), st);
         if (e != cudaSuccess) return e;
         const int64_t na = distinct_items(g.a_is, g.a_div, g.n_items), nb_ = distinct_items(g.b_is, g.b_div, g.n_items);
+        // a grid-stride loop: 8 CTAs for each of a GB300's 152 SMs are enough to fill them
         auto blocks = [](int64_t entries) { return (unsigned)std::min<int64_t>((entries / 2 + 255) / 256, 152 * 8); };
         k_absmax<<<blocks(M * K * na), 256, 0, st>>>(g.a, g.a_is, g.mb + g.kb, na, g.amax);
         k_absmax<<<blocks(N * K * nb_), 256, 0, st>>>(g.b, g.b_is, g.nb + g.kb, nb_, g.amax + 1);
