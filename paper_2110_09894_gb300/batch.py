@@ -6,9 +6,9 @@ Members whose intermediates fit one CTA's scratch (at most 2^18 entries per
 (slice, bitstring) pair, no tensor-core step) form a group of the C ABI
 (qx_group_*): those with little work per pair run in its persistent launch
 (whole contractions per CTA, one FP64 sum), the group runs the others as
-launches over batches of pairs in its scratch; the heavy members -- large intermediates, tensor-core products -- run on the batched
-executor (one launch per step over many pairs, steps at their dependence
-level).  Everything is enqueued on one stream and captured as one CUDA graph,
+launches over batches of pairs in its scratch.  The heavy members -- large
+intermediates, tensor-core products -- run on the batched executor (one
+launch per step over many pairs, steps at their dependence level).  Everything is enqueued on one stream and captured as one CUDA graph,
 so a step of the whole workload is one graph launch.
 
 Only argument marshalling lives here: every step runs in libqx's kernels.
