@@ -344,9 +344,13 @@ def group_bench(args):
             checked += 1
         parity = {"vs": "complex128 state vectors (batched_statevector.json)", "members_checked": checked,
                   "worst_rel_l2": worst_l2, "worst_max_elem_over_rms": worst_el}
+    n_light, n_heavy = len(b.light), len(b.heavy)
     # the same members in plain complex64 (heavy members on the SIMT kernels), same settings
     vs_c64 = None
     if prec != 0 and not args.no_forms:
+        b.close()  # both workspaces don't fit side by side
+        del b
+        torch.cuda.empty_cache()
         b64 = UnevenBatch(ws, precision=0, ctas_per_sm=choice["ctas_per_sm"],
                           settings={int(i): s for i, s in choice["settings"].items()})
         b64.capture()
@@ -356,7 +360,6 @@ def group_bench(args):
                   "worst_rel_diff_to_c64": max(float(np.linalg.norm(x - y) / np.linalg.norm(y))
                                                for x, y in zip(got, a64))}
         b64.close()
-    n_light, n_heavy = len(b.light), len(b.heavy)
     line = {"metric": "amplitudes/s", "value": amps * len(ms) / (sum(ms) / 1e3), "unit": "amplitudes/s",
             "n_gpus": 1, "steps": args.steps, "warmup": args.warmup, "ms_per_step": sum(ms) / len(ms),
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
