@@ -349,7 +349,7 @@ def group_bench(args):
     vs_c64 = None
     if prec != 0 and not args.no_forms:
         b.close()  # both workspaces don't fit side by side
-        del b
+        b = None
         torch.cuda.empty_cache()
         b64 = UnevenBatch(ws, precision=0, ctas_per_sm=choice["ctas_per_sm"],
                           settings={int(i): s for i, s in choice["settings"].items()})
@@ -376,7 +376,8 @@ def group_bench(args):
             "complex_tflops_executed": flops * len(ms) / (sum(ms) / 1e3) / 1e12, "parity": parity,
             "graph_replay_equals_eager_run": replay_equal, "vs_plain_c64": vs_c64,
             "gpu_launches": int(launches * args.steps), "clocks": clocks}
-    b.close()
+    if b is not None:
+        b.close()
     print(json.dumps(line), flush=True)
 
 
