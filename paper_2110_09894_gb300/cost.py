@@ -13,8 +13,8 @@ steps of a seg= number) where the library runs it so, by the library's own
 rule.  The rates were measured per family on the 36-qubit sliced workload.  Against
 calls on one stream, as a serving lane makes them (31 calls of 33 us to 74 ms:
 the benchmark's and seven serving plans, 1 to 1024 bitstrings), the sums lie at
-0.81 to 1.37 of the measured times.  With concurrent streams the calls whose
-launches are short take down to 0.55 of the estimate.
+0.81 to 1.39 of the measured times.  With concurrent streams the calls whose
+launches are short take down to 0.5 of the estimate.
 The server uses the estimate for admission, planners to rank plans.
 """
 from __future__ import annotations
@@ -27,6 +27,7 @@ GB300_LAUNCH_RATES = {"permute": (None, 6.0e12), "gather": (26e12, 4.7e12), "tc_
 _LEVEL = {"shared": 0, "slice": 1, "pair": 2}
 _SM, _CLOCK, _WARPS = 152, 1.9e9, 4  # SMs, their clock, warps that an SM issues from at a time
 _TILE16 = 64e9  # complex flop/s of the GEMM on one SM, on the 16 x 16 tiles of a product with few outputs
+_SHORT = 16e12  # complex flop/s of the GEMM with a short side of at most 4
 _BANKS = 3.5  # issue time of a segment against its listed clocks (shared-memory bank conflicts)
 
 
@@ -55,6 +56,8 @@ def _step_time(kind, level, kv, items, rates):
     t = nbytes / br
     if fr and "m" in kv:
         m, k, n = int(kv["m"]), int(kv["k"]), int(kv["n"])
+        if kind == "gemm" and min(m, n) <= 2:
+            fr = min(fr, _SHORT)
         t = max(t, 8.0 * 2.0 ** (m + k + n) * it / fr)
         # few tiles: one tile's sum over K on its SM (128 x 64 on the tensor cores; the GEMM takes tiles of
         # 16 x 16 then)
@@ -72,19 +75,23 @@ def _segment_time(kv, n_items, sms=_SM):
                _BANKS * n_items * float(kv["clocks"]) / (sms * _WARPS) / _CLOCK)
 
 
+def parse(desc):
+    """The steps of a qx_describe_plan listing: (kernel family, dependence level, fields)."""
+    rows = (line.split() for line in desc.splitlines())
+    return [(f[2], f[3], dict(x.split("=", 1) for x in f[4:] if "=" in x)) for f in rows]
+
+
 def launches(desc, items, rates=GB300_LAUNCH_RATES, launch=4e-6):
-    """(dependence level, seconds) of every launch of a batch from a qx_describe_plan listing; items: the
-    launches' items by level (1, slices, (slice, bitstring) pairs)."""
+    """(dependence level, seconds) of every launch of a batch from a qx_describe_plan listing (or its
+    parsed steps); items: the launches' items by level (1, slices, (slice, bitstring) pairs)."""
     out, chains, segs = [], [], {}
-    for line in desc.splitlines():
-        f = line.split()
-        kv = dict(x.split("=", 1) for x in f[4:] if "=" in x)
-        level = _LEVEL[f[3]]
+    for kind, name, kv in parse(desc) if isinstance(desc, str) else desc:
+        level = _LEVEL[name]
         if "chain" in kv:  # all chains run in one launch, a CTA each
             if "stages" in kv:
                 chains.append(_segment_time(kv, 1, 1))
             continue
-        t = _step_time(f[2], f[3], kv, items, rates) + launch
+        t = _step_time(kind, name, kv, items, rates) + launch
         if "seg" not in kv:
             out.append((level, t))
             continue
@@ -100,9 +107,14 @@ def launches(desc, items, rates=GB300_LAUNCH_RATES, launch=4e-6):
     return out
 
 
-def launch_list_time(desc, n_slices, n_bits, rates=GB300_LAUNCH_RATES, launch=4e-6):
-    """Seconds of one call over n_slices slices and n_bits bitstrings from a qx_describe_plan listing
-    (launches priced one after another), with the launches that every call has: two clears, the sum over
-    the slices (0.3 us each, in order) and its end."""
-    return sum(t for _, t in launches(desc, (1, n_slices, n_slices * n_bits), rates, launch)) + \
-        4 * launch + 0.3e-6 * n_slices
+def launch_list_time(desc, n_slices, n_bits, rates=GB300_LAUNCH_RATES, launch=4e-6, max_items=None, kept=False):
+    """Seconds of one call over n_slices slices and n_bits bitstrings from a qx_describe_plan listing (or
+    its parsed steps; launches priced one after another), with the launches that every call has: two
+    clears, the sums over the slices (0.3 us each, in order) and their end.  max_items: (slice, bitstring)
+    pairs that a batch of the workspace holds, at least n_bits of them; None: all.  kept: the invariant
+    intermediates are kept from an earlier call (qx_set_memo)."""
+    per = n_slices if max_items is None else max(1, min(n_slices, max_items // n_bits))
+    batches = -(-n_slices // per)
+    listed = launches(desc, (1, per, per * n_bits), rates, launch)
+    once, per_batch = (sum(t for level, t in listed if (level > 0) == later) for later in (False, True))
+    return (0.0 if kept else once) + batches * (per_batch + launch) + 3 * launch + 0.3e-6 * n_slices

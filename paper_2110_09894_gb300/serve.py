@@ -29,7 +29,8 @@ while other work is on the GPU:
   offered load beyond the GPU, admitted requests keep a bounded latency
   instead of every request waiting in an unbounded queue).  Service times
   are estimated from the library's compiled launch list of the circuit's
-  plan (cost.launch_list_time), linear in the number of bitstrings.
+  plan (cost.launch_list_time) in the lane's batches, with the invariant
+  intermediates kept.
 
 The scheduling runs on the host in Python (it only marshals work); every
 contraction step runs in the library's kernels.
@@ -43,7 +44,7 @@ from dataclasses import dataclass, field
 import numpy as np
 
 from . import qx
-from .cost import launch_list_time, launches
+from .cost import launch_list_time, parse
 
 
 @dataclass
@@ -100,11 +101,9 @@ class ServedCircuit:
     n_slices: int = 1
     lane_bytes: int = 0
     servable: bool = True
-    est_a: float = 0.0          # estimated seconds of one batch of b bitstrings: est_a + est_b * b
-    est_b: float = 0.0
+    est_bits: tuple = (1,)      # estimated seconds of a piece by its bitstrings, linear in between
+    est_s: tuple = (0.0,)       # (with the invariant intermediates kept, as from a lane's first request on)
     items: int = 1              # (slice, bitstring) pairs per batch in a lane's workspace
-    slice_ops: int = 0          # launches per batch of the per-slice and the per-pair steps
-    pair_ops: int = 0
 
     def piece(self, n_bits):
         """Bitstrings per piece of a request: a lane runs a request as pieces of at most one batch of
@@ -112,17 +111,12 @@ class ServedCircuit:
         work."""
         return max(1, min(n_bits, self.items))
 
-    def estimate(self, n_bits, launch_s=1e-5):
-        """Estimated seconds of a request: per piece its work (whole slices with all the piece's
-        bitstrings per batch, the launches of every extra batch counted) and its fixed part."""
-        total, left = 0.0, n_bits
-        while left > 0:
-            pn = self.piece(left)
-            per = max(1, self.items // pn)
-            extra = (-(-self.n_slices // per) - 1) * (self.slice_ops + self.pair_ops)
-            total += self.est_a + self.est_b * pn + extra * launch_s
-            left -= pn
-        return total
+    def estimate(self, n_bits):
+        """Estimated seconds of a request: the sum over its pieces, each in batches of whole slices with all
+        the piece's bitstrings."""
+        whole, rest = divmod(n_bits, self.piece(n_bits))
+        total = whole * np.interp(self.piece(n_bits), self.est_bits, self.est_s)
+        return float(total + (np.interp(rest, self.est_bits, self.est_s) if rest else 0.0))
     lanes: list = field(default_factory=list)
     queue: collections.deque = field(default_factory=collections.deque)
 
@@ -160,12 +154,10 @@ class Server:
             sc.items = items
             sc.lane_bytes = qx.qx_workspace_size(h, max_bits, items)
             sc.servable = sc.lane_bytes <= self.budget
-            desc = qx.qx_describe_plan(h)
-            lv = [level for level, _ in launches(desc, (1, min(sc.n_slices, items), items))]
-            sc.slice_ops, sc.pair_ops = lv.count(1), lv.count(2)
-            t1 = launch_list_time(desc, sc.n_slices, 1)
-            sc.est_b = max((launch_list_time(desc, sc.n_slices, 256) - t1) / 255.0, 0.0)
-            sc.est_a = t1 - sc.est_b
+            steps = parse(qx.qx_describe_plan(h))
+            most = min(items, max_bits)
+            sc.est_bits = tuple(sorted({1 << k for k in range(most.bit_length())} | {most}))
+            sc.est_s = tuple(launch_list_time(steps, sc.n_slices, b, max_items=items, kept=True) for b in sc.est_bits)
             qx.qx_destroy(h)
             self.circuits.append(sc)
         self.clock0 = time.perf_counter()

@@ -47,6 +47,25 @@ def test_estimates_lie_near_the_measured_times(plan, n_bits, measured_us):
     assert measured_us / 1.5 < est < 1.5 * measured_us
 
 
+@pytest.mark.parametrize("j,precision,n_bits,items,measured_ms", [
+    (9, 1, 1, 1024, 0.20), (9, 1, 300, 1024, 6.52), (3, 0, 40, 185, 1.84), (6, 0, 40, 101, 6.85),
+    (7, 1, 300, 658, 0.89), (6, 1, 102, 102, 3.83)])
+def test_a_lanes_piece_is_priced_in_its_batches_with_kept_invariants(j, precision, n_bits, items, measured_ms):
+    """Requests on an idle server after the lane's first one (host time among it)."""
+    desc, n_slices = _served(j, precision)
+    est = 1e3 * cost.launch_list_time(desc, n_slices, n_bits, max_items=items, kept=True)
+    assert measured_ms / 1.5 < est < 1.5 * measured_ms
+    assert cost.launch_list_time(desc, n_slices, n_bits, max_items=items) > est / 1e3
+
+
+def test_batches_of_a_sliced_call_repeat_its_per_batch_launches():
+    desc, n_slices = _sliced(1)
+    whole = cost.launch_list_time(desc, n_slices, 16)
+    assert cost.launch_list_time(desc, n_slices, 16, max_items=16 * n_slices) == whole
+    half = cost.launch_list_time(desc, n_slices, 16, max_items=16 * n_slices // 2)
+    assert whole < half < 2 * whole
+
+
 def test_a_segment_is_one_launch_where_it_runs_as_one():
     desc, n_slices = _sliced(1)
     seg = {m[1] for m in re.finditer(r" seg=(\d+)", desc)}
