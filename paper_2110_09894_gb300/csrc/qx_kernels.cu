@@ -760,8 +760,8 @@ __global__ void __launch_bounds__(256, 2) k_gemm_c64(const float2* __restrict__ 
 // ---------------------------------------------------------------------------------------------
 // The same GEMM on packed FP32 FMAs (fma.rn.f32x2), for M, N >= 32 and K >= 8.  An FMA with three
 // different register operands issues at 0.7 of the FP32 rate here (57 of 80 TFLOP/s in a register-only
-// loop; packed 64), and a complex multiply-add takes four, so k_gemm_c64 filled its issue slots (80%,
-// FMA pipe 56%) at 30 to 47 TFLOP/s.  Packed, a multiply-add is two instructions on (re, im) sums,
+// loop; packed 64), and a complex multiply-add takes four, so k_gemm_c64 is bound by its issue slots at 30
+// to 47 TFLOP/s.  Packed, a multiply-add is two instructions on (re, im) sums,
 //     acc += (ar, ar) * (br, bi),   acc += (ai, ai) * (-bi, br),
 // the same four roundings in the same order.  The operands stay 8 bytes in shared memory and are
 // doubled in registers: reading them doubled (16 bytes) costs 48 clocks of the load path per k and
@@ -769,7 +769,8 @@ __global__ void __launch_bounds__(256, 2) k_gemm_c64(const float2* __restrict__ 
 // side) per CTA, 8 x 4 per thread, 8 k per stage, register-staged double buffer; 64 x 64 rather than
 // 128 x 64 so that several CTAs per SM cover each other's barriers.  FOLD (K > 64): sums of 64 k are
 // added to running totals (see above), kept in shared memory so that the registers hold three CTAs
-// per SM; shorter sums need no total.  Now bound by the packed FMAs' operand reads (pipe 67% busy).
+// per SM; shorter sums need no total.  Bound by the packed FMAs' operand reads: FMA pipe 66% busy, math
+// pipe throttle the first stall (M = N = 128, K = 64, 600 items: 110 us).
 // Before / after (us): 64 x 128 x 64 for 16384 items 1571 / 1420; 32 x 256 x 64 for 16384 1898 / 1428;
 // 2048 x 512 x 512 for 64 5897 / 5409; 2^15 x 32 x 32 for 64 545 / 371; 256 x 512 x 8 for 1024 455 / 261.
 // ---------------------------------------------------------------------------------------------
