@@ -89,7 +89,11 @@ typedef struct {
                                 may store products in the layout the next
                                 GEMM reads and fuse the last permute into the
                                 dot, which only the batched launches do, so
-                                set 2 or 3 before qx_set_plan */
+                                set 2 or 3 before qx_set_plan.  A workspace
+                                holds the regions of the executor it was
+                                bound for: after a change, bind it again
+                                (else QX_ESTATE for 2, QX_ENOMEM for a
+                                member's workspace without batch regions) */
     int64_t timeout_cycles;  /* bound on each device spin-wait, in SM clock
                                 cycles; 0 = default (2e9).  An expired wait
                                 makes the call report QX_ETIMEOUT (through
@@ -248,7 +252,8 @@ int qx_set_graphs(qx_handle h, int enable);
  * (the kept tensors are the ones the skipped steps would write again).
  * enable = 0 (default): every call computes them.  qx_contract_device_static
  * always computes them.  A device timeout reported by qx_device_status
- * drops the kept tensors.  Drops a captured graph.  QX_EINVAL unless enable
+ * drops the kept tensors and the captured graphs; a call that is only being
+ * captured leaves none behind.  Drops a captured graph.  QX_EINVAL unless enable
  * is 0 or 1. */
 int qx_set_memo(qx_handle h, int enable);
 
@@ -273,7 +278,8 @@ int qx_set_streams(qx_handle h, int32_t n_streams);
  * whether it runs per pair or once, M/K/N bits, operand layouts).  Steps with
  * the same chain= or seg= number may run as one launch: chains in the
  * prologue launch of a call, segments where one launch is the faster way for
- * the call's items.  Writes at most len bytes (NUL-terminated) to buf; *needed (may be
+ * the call's items (its last step lists what that rule weighs: stages, issue
+ * clocks per item, bytes per item of launches per step).  Writes at most len bytes (NUL-terminated) to buf; *needed (may be
  * NULL) receives the full size.  Works on host-only handles. */
 int qx_describe_plan(qx_handle h, char* buf, int64_t len, int64_t* needed);
 
