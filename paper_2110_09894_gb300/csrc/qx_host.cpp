@@ -168,6 +168,7 @@ struct qx_ctx : Offsets {
         int n_stages = 0, n_tasks = 0, arena = 0;
         double warp_clocks = 0;        // estimated issue clocks of one item's tasks
         double bytes = 0;              // of its steps as launches of their own, per item
+        double moved[3] = {0, 0, 0};   // bytes of its operands from outside and its result, by their level
         double flops = 0;
         int64_t prog_off = 0;          // bytes into seg_blob
         int32_t prog_bytes = 0;
@@ -182,7 +183,7 @@ struct qx_ctx : Offsets {
     std::vector<std::pair<int64_t, int64_t>> pair_life;  // their lifetimes when a CTA runs one pair's steps in order
     bool wave_ok = false;               // there is a prologue launch
     std::vector<int> chain_of_op;       // per op: its prologue segment, -1 if none
-    double wave_flops = 0;
+    double wave_flops = 0, wave_bytes = 0;
     bool segs_on_device = false;
     cudaEvent_t wave_ev = nullptr;
 
@@ -1732,7 +1733,7 @@ static void build_segments(qx_ctx* h) {
     h->seg_blob.clear();
     h->n_waves = 0;
     h->wave_ok = false;
-    h->wave_flops = 0;
+    h->wave_flops = h->wave_bytes = 0;
     h->chain_of_op.assign(h->ops.size(), -1);
     std::vector<int32_t> wave_offs;
     for (auto& sg : h->segs) {
@@ -1747,11 +1748,13 @@ static void build_segments(qx_ctx* h) {
             in.once = t.once;
             in.natural = 1;
             const int sid = seg_storage(h, op, t.side);
+            const int node = op.type == OP_GEMM ? -1 : op.type == OP_PERM ? op.src : t.side ? op.y : op.x;
+            sg.moved[sid >= 0 ? h->stor[sid].level : h->nodes[node].level] += 8.0 * (double)((int64_t)1 << t.bits);
             if (sid >= 0) {
                 in.off = h->stor[sid].off;
                 in.space = h->stor[sid].level;
             } else {
-                const Node& nd = h->nodes[op.type == OP_PERM ? op.src : t.side ? op.y : op.x];
+                const Node& nd = h->nodes[node];
                 in.off = nd.leaf_off;
                 in.space = SEG_LEAF;
                 for (int b = 0; b < in.rank; ++b) {
@@ -1853,6 +1856,7 @@ static void build_segments(qx_ctx* h) {
         hd.n_tiny = p.n_tiny;
         hd.arena = p.arena;
         const Storage& out = h->stor[h->ops[sg.ops.back()].dst];
+        sg.moved[out.level] += 8.0 * (double)out.entries;
         hd.out_space = out.level;
         hd.out_entries = (int32_t)out.entries;
         hd.out_off = out.off;
@@ -1876,6 +1880,7 @@ static void build_segments(qx_ctx* h) {
             for (int i : sg.ops) h->chain_of_op[i] = h->n_waves;
             wave_offs.push_back((int32_t)sg.prog_off);
             h->wave_flops += sg.flops;
+            h->wave_bytes += sg.moved[0];
             h->n_waves++;
         }
     }
@@ -1928,13 +1933,9 @@ static double op_bytes(const qx_ctx* h, const Op& op, int64_t n_items, int64_t n
 // Bytes that a segment's launch moves: the operands from outside it and the result (the steps' other
 // tensors stay in shared memory; op_bytes counts those of launches per step)
 static double seg_traffic(const qx_ctx* h, const qx_ctx::Seg& sg, int64_t n_items, int64_t n_b = 1) {
-    double bytes = 8.0 * (double)h->stor[h->ops[sg.ops.back()].dst].entries * (double)n_items;
-    for (const auto& t : sg.plan->in) {
-        const Op& op = h->ops[sg.ops[t.op]];
-        const int sid = seg_storage(h, op, t.side);
-        const int level = sid >= 0 ? h->stor[sid].level : h->nodes[op.type == OP_PERM ? op.src : t.side ? op.y : op.x].level;
-        bytes += 8.0 * (double)((int64_t)1 << t.bits) * copies(op, level, n_items, n_b);
-    }
+    const Op& root = h->ops[sg.ops.back()];
+    double bytes = 0;
+    for (int level = 0; level < 3; ++level) bytes += sg.moved[level] * copies(root, level, n_items, n_b);
     return bytes;
 }
 
@@ -2230,15 +2231,13 @@ struct Dag {
         SegCtx c = seg_ctx(ic, 1, 0);
         c.prog = (const uint8_t*)(h->ws + h->off_wave);
         c.prog_off = (const int32_t*)(c.prog + h->wave_list);
-        double bytes = 0;
         for (const auto& sg : h->segs)
             if (sg.wave) {
-                bytes += seg_traffic(h, sg, 1);
                 c.prog_bytes = std::max(c.prog_bytes, sg.prog_bytes);
                 c.arena = std::max(c.arena, sg.arena);
             }
         size_t slot;
-        cudaError_t e = prof_begin(h, QX_KERNEL_WAVE, h->wave_flops, bytes, &slot);
+        cudaError_t e = prof_begin(h, QX_KERNEL_WAVE, h->wave_flops, h->wave_bytes, &slot);
         if (e == cudaSuccess) e = launch_seg(c, h->n_waves, 512, h->stream);
         if (e == cudaSuccess) e = prof_end(h, slot);
         if (e == cudaSuccess && on) e = cudaEventRecord(h->wave_ev, h->stream);
