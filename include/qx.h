@@ -396,7 +396,9 @@ int qx_esup_sample(qx_handle h, const uint8_t* d_candidates, const double* d_uni
  *                    steps once per slice.  The amplitudes are the same
  *                    either way.  No allocation, no host copies, no
  *                    synchronisation, so a CUDA graph can capture it.
- * A group does not own its members; destroy it before them. */
+ * A group does not own its members; destroy it before them.  A run uses the
+ * members' handles and workspaces: calls on a member, or runs of another group
+ * that holds it, must not overlap it, on the host or on the device. */
 typedef struct qx_group* qx_group_t;
 int qx_group_create(qx_group_t* g, qx_handle* hs, int32_t n, const uint8_t* const* d_bitstrings,
                     const int64_t* n_bits, double* const* d_amps_out, int32_t ctas_per_sm);

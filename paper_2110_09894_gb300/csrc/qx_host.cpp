@@ -2725,6 +2725,7 @@ int qx_bind_workspace_parts(qx_handle h, void* d_fixed, int64_t fixed_bytes, voi
     if (!d_fixed || !d_batch) return fail(h, QX_EINVAL, "null buffer");
     if (((uintptr_t)d_fixed) % 256 || ((uintptr_t)d_batch) % 256)
         return fail(h, QX_EINVAL, "workspace parts must be 256-byte aligned");
+    if (h->opt.executor >= 2) persist_program(h);
     if (persist_member(h) || persist_active(h))
         return fail(h, QX_EINVAL, "a split workspace is for the batched executor");
     unbind(h);

@@ -64,3 +64,19 @@ def test_the_persistent_executor_needs_a_workspace_bound_for_it(qx):
     qx.qx_set_options(c.h)  # and back: the batched regions are part of it
     assert_parity(c.contract(bits), ref)
     c.close()
+
+
+def test_a_split_workspace_stays_refused_for_the_persistent_executors(qx):
+    import torch
+    circ, om, order, sliced, _ = grid_case(2, 3, 4, 7, 0, 0, 3)
+    for first, then in ((0, 2), (0, 3), (2, 2), (3, 3)):
+        h = qx.qx_create(0, executor=first)
+        qx.qx_build_network(h, circ.n_qubits, C.gates_to_records(circ), om)
+        qx.qx_set_plan(h, order, sliced)
+        qx.qx_set_options(h, executor=then)
+        fixed = torch.empty(1 << 20, dtype=torch.uint8, device="cuda")
+        batch = torch.empty(1 << 20, dtype=torch.uint8, device="cuda")
+        with pytest.raises(qx.QXError) as e:
+            qx.qx_bind_workspace_parts(h, fixed.data_ptr(), 1 << 20, batch.data_ptr(), 1 << 20, 3)
+        assert e.value.code == qx.QX_EINVAL
+        qx.qx_destroy(h)
